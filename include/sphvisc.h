@@ -111,9 +111,12 @@ typedef struct sph_neighbors sph_neighbors;
  * the float32 positions (a float32 test with a safety band, then a float64
  * recheck inside the band).
  * max_neighbors: capacity per particle, 1..1024; a larger count returns
- *   SPH_ERR_CAPACITY.  The lists are built in one pass into a layout of that
- *   capacity: 4 * max_neighbors bytes of device memory per particle (512 B at
- *   the default 128).
+ *   SPH_ERR_CAPACITY.  The lists are kept in a layout of that capacity as 16-bit
+ *   positions among the distinct neighbours of a run of rows: about
+ *   4 * max_neighbors bytes of device memory per particle with the search's own
+ *   copy (520 B at the default 128).  Particle sets too uneven for that, and the
+ *   entry points that walk 32-bit rows (export, the on-the-fly apply, features),
+ *   take 4 * max_neighbors bytes more.
  * Copies pos/rho/mu/ptype into the handle: the scene arrays may be freed after
  * the call returns. */
 sph_status sph_build_neighbors(const sph_scene* scene, int32_t max_neighbors,
@@ -236,8 +239,9 @@ typedef struct {
   int32_t jacobi;          /* 1: Jacobi scaling (App. B): left scaling of the
                               BiCGSTAB system, z = D^-1 r in the CG; 0: none
                               (CG only: BiCGSTAB returns SPH_ERR_INVALID)        */
-  int32_t apply_form;      /* 0: the autotuner picks the operator apply's row-loop
-                              form per phase (default); k = 1..6: use form k - 1
+  int32_t apply_form;      /* 0: the tile form, or where the lists have none the
+                              autotuner's choice of row-loop form per phase
+                              (default); k = 1..6: use form k - 1
                               (sph_profile_counters.apply_variant numbering)     */
   int32_t launch_mode;     /* 0: the BiCGSTAB loop's kernels are programmatic
                               dependent launches, each launch processed while its
@@ -707,7 +711,11 @@ typedef struct {
                                 in registers; 4 = coefficient stream staged in shared
                                 memory by bulk asynchronous copies; 5 = each 32-row
                                 slice's distinct neighbour vectors gathered once into
-                                shared memory                                        */
+                                shared memory; 6 = the tile form (16-bit positions
+                                among a run of rows' distinct neighbours, those
+                                vectors in shared memory), which needs no tuning and
+                                is taken whenever the lists have it and no form is
+                                asked for                                            */
   float tune_us[3][6];       /* autotuner timings (us) per phase (A p, A r*, A r* with
                                 merged dots) and form; 0 where not measured          */
   int64_t standalone_launches[2]; /* sph_visc_apply [0] and sph_visc_apply_otf [1] calls

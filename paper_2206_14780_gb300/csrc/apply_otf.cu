@@ -162,6 +162,7 @@ __global__ void k_scatter_f4_otf(const float4* __restrict__ y_s, const int32_t* 
 // with the stored operator: same dt, boundary, mean and viscosities).
 static sph_status ensure_otf(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st) {
   SPH_TRY(ensure_operator(H, P, st));
+  SPH_TRY(ensure_nbr(H, st));
   if (H->otf_valid && H->otf_op_version == H->op_version) return SPH_OK;
   SPH_TRY(H->otf_g.alloc(H->n_pad));
   SPH_TRY(H->otf_im.alloc(H->n_pad));

@@ -667,7 +667,7 @@ sph_status sph_batch_create(sph_neighbors* const* handles, const sph_visc_params
       set_error("sph_batch_create: handle %d is null", s);
       return fail(SPH_ERR_INVALID);
     }
-    sph_status e = ensure_operator(H, &params[s], st);
+    sph_status e = ensure_operator(H, &params[s], st, OP_IH);
     if (e == SPH_OK) e = row_scale_refresh(H, st);
     if (e != SPH_OK) return fail(e);
     Bt->handles.push_back(H);

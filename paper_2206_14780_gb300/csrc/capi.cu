@@ -134,6 +134,19 @@ sph_status sph_neighbors_destroy(sph_neighbors* h) {
   h->cnt.release();
   h->slice_off.release();
   h->nbr.release();
+  h->t_idx.release();
+  h->t_raw.release();
+  h->t_cells.release();
+  h->t_ncell.release();
+  h->t_unum.release();
+  h->t_uni.release();
+  h->t_nfl.release();
+  h->t_off.release();
+  h->t_hi.release();
+  h->t_lo.release();
+  h->t_nnz.release();
+  h->tmp_ids.release();
+  h->scan_sums.release();
   h->op_cnt.release();
   h->op_off.release();
   h->op_ih.release();
@@ -357,6 +370,12 @@ sph_status sph_profile_read(sph_neighbors* h, sph_profile_counters* out, int32_t
   if (h) {
     out->apply_launches = h->prof_n;
     out->apply_ms = h->prof_ms;
+    if (h->op_nnz < 0) {   // counted by the tile fill on the device
+      unsigned long long c = 0;
+      SPH_TRY_CUDA(cudaDeviceSynchronize());
+      SPH_TRY_CUDA(cudaMemcpy(&c, h->t_nnz.p, sizeof(c), cudaMemcpyDeviceToHost));
+      h->op_nnz = (int64_t)c;
+    }
     out->op_nnz = h->op_nnz;
     out->apply_bytes = 8 * h->op_nnz + (16 + 16 + 16 + 9) * h->n;
     for (int k = 0; k < 2; ++k) {
@@ -365,6 +384,7 @@ sph_status sph_profile_read(sph_neighbors* h, sph_profile_counters* out, int32_t
     }
     out->apply_variant[0] = h->apply_var[0];
     out->apply_variant[1] = h->apply_var[1] > h->apply_var[2] ? h->apply_var[1] : h->apply_var[2];
+    if (h->tile_grid > 0) out->apply_variant[0] = out->apply_variant[1] = kApplyVariants;
     for (int ph = 0; ph < 3; ++ph)
       for (int v = 0; v < kApplyVariants; ++v) out->tune_us[ph][v] = h->tune_us[ph][v];
     for (int f = 0; f < 2; ++f) {
@@ -374,6 +394,7 @@ sph_status sph_profile_read(sph_neighbors* h, sph_profile_counters* out, int32_t
     out->otf_bytes = 4 * h->nnz + (16 + 16 + 16 + 4 + 4 + 4 + 1) * h->n;
     out->apply_grid[0] = h->apply_grid[0];
     out->apply_grid[1] = h->apply_grid[1] > 0 ? h->apply_grid[1] : h->apply_grid[2];
+    if (h->tile_grid > 0) out->apply_grid[0] = out->apply_grid[1] = h->tile_grid;
     if (reset) {
       h->prof_n = 0;
       h->prof_ms = 0.0;

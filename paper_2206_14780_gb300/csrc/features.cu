@@ -416,6 +416,7 @@ __global__ void k_resid_targets(const float4* __restrict__ y, const float4* __re
 sph_status features_impl(sph_neighbors* H, const sph_visc_params* P, const float* vel, __nv_bfloat16* feats,
                          cudaStream_t st, bool walls_only) {
   SPH_TRY(ensure_operator(H, P, st));
+  SPH_TRY(ensure_nbr(H, st));
   SPH_TRY(ensure_workspace(H));
   SPH_TRY(H->feat_tmp.alloc(4 * H->n_pad));
   SPH_TRY(H->feat_scale.alloc(2));
@@ -427,9 +428,9 @@ sph_status features_impl(sph_neighbors* H, const sph_visc_params* P, const float
   const int grid = grid_for(H, np);
   SPH_LAUNCH(k_feat_gather, grid, kBlock, 0, st)(reinterpret_cast<const float4*>(vel), H->perm.p, H->n, np, vs);
   if (!walls_only) {
-    launch_apply_f32(H, vs, y, false, st);
+    launch_apply_f32(H, vs, y, st);
     SPH_LAUNCH(k_feat_incr, grid, kBlock, 0, st)(vs, y, H->invD.p, H->type_s.p, H->n, np, e1);
-    launch_apply_f32(H, e1, y, false, st);
+    launch_apply_f32(H, e1, y, st);
     SPH_LAUNCH(k_feat_incr, grid, kBlock, 0, st)(e1, y, H->invD.p, H->type_s.p, H->n, np, e2);
   }
   int rg = grid < H->red_grid ? grid : H->red_grid;
@@ -457,11 +458,15 @@ sph_status features_impl(sph_neighbors* H, const sph_visc_params* P, const float
 // x0 (caller order, device double [n][3]) gets its dummy-wall rows from Eq.
 // dummyvel given its fluid rows; uses feat_tmp slots 0 and 1
 static void wall_closure(sph_neighbors* H, double* x0, const double* b, cudaStream_t st) {
+  if (H->op_tile_valid) {
+    tile_wall_close(H, x0, b, st);
+    return;
+  }
   const int64_t np = H->n_pad;
   float4* xs = H->feat_tmp.p;
   float4* ax = xs + np;
   SPH_LAUNCH(k_x0_sorted, grid_for(H, np), kBlock, 0, st)(x0, H->perm.p, H->type_s.p, 1, H->n, np, xs);
-  launch_apply_f32(H, xs, ax, false, st);
+  launch_apply_f32(H, xs, ax, st);
   SPH_LAUNCH(k_wall_close, grid_for(H, H->n), kBlock, 0, st)(ax, b, H->perm.p, H->type_s.p, H->n, x0);
 }
 
@@ -636,12 +641,12 @@ sph_status sph_mlp_residual_targets(sph_neighbors* h, const sph_visc_params* par
   float4* z = xs + 2 * np;
   float4* az = xs + 3 * np;
   SPH_LAUNCH(k_x0_sorted, grid_for(h, np), kBlock, 0, st)(x0, h->perm.p, h->type_s.p, 0, h->n, np, xs);
-  launch_apply_f32(h, xs, ax, false, st);
+  launch_apply_f32(h, xs, ax, st);
   const int rg = grid_for(h, np) < h->red_grid ? grid_for(h, np) : h->red_grid;
   double* sums = h->r64.p;
   SPH_LAUNCH(k_resid_z, rg, kBlock, 0, st)(ax, b, h->perm.p, h->type_s.p, h->invD.p, (flags & SPH_RLOSS_JACOBI) ? 1 : 0,
                                            h->n, np, z, h->partials.p, h->counters.p + 7, sums);
-  launch_apply_f32(h, z, az, false, st);
+  launch_apply_f32(h, z, az, st);
   const float4* grad = az;
   if (hp) {                           // P^T = I - S^T in front of A z (slot 0 is free again)
     highpass_T(h, az, h->feat_den.p, xs, st);

@@ -99,7 +99,7 @@ sph_status visc_apply_noalloc(sph_neighbors* H, const sph_visc_params* P, const 
   const int grid = grid_for(H, H->n_pad);
   SPH_LAUNCH(k_na_gather, grid, kBlock, 0, st)(reinterpret_cast<const float4*>(v), H->perm.p, H->n, H->n_pad, vs);
   SPH_TRY_CUDA(cudaGetLastError());
-  launch_apply_f32(H, vs, ys, false, st);
+  launch_apply_f32(H, vs, ys, st);
   SPH_TRY_CUDA(cudaGetLastError());
   SPH_LAUNCH(k_na_scatter, grid, kBlock, 0, st)(ys, H->perm.p, H->n, reinterpret_cast<float4*>(y));
   SPH_TRY_CUDA(cudaGetLastError());

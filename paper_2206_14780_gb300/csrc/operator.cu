@@ -19,20 +19,14 @@
 #include "apply.cuh"
 #include "dfloat.cuh"
 #include "reduce.cuh"
+#include "pair_df.cuh"
 #include "residual_row.cuh"
 #include "sph_internal.cuh"
+#include "tiles.cuh"
 
 namespace sph {
 
 namespace {
-
-struct OpGeom {
-  double L[3];
-  double invL[3];
-  int periodic[3];
-  double h;
-  double inv_h;
-};
 
 // per particle: V = m / rho and 1 / mu, evaluated in float64 once per particle
 // and kept as double-float pairs (V hi, V lo, 1/mu hi, 1/mu lo)
@@ -43,58 +37,6 @@ __global__ void k_op_aux(const float4* __restrict__ pos, const float* __restrict
     const dfl im = df_from_double(1.0 / (double)mu[s]);
     aux[s] = make_float4(V.hi, V.lo, im.hi, im.lo);
   }
-}
-
-// Geometry of the double-float set-up: periods as (hi, lo), 1/h as (hi, lo)
-struct OpGeomDF {
-  dfl L[3];
-  float invL[3];
-  int periodic[3];
-  dfl inv_h;
-};
-
-// |r_a - r_b| in double-float: the coordinate differences of the float32
-// positions exactly (TwoSum), the minimum image by a whole period, the squared
-// norm with exact products, one Newton step on the root
-__device__ __forceinline__ dfl pair_r_df(float4 pa, float4 pb, const OpGeomDF& g) {
-  dfl d[3] = {df_exact_sum(pa.x, -pb.x), df_exact_sum(pa.y, -pb.y), df_exact_sum(pa.z, -pb.z)};
-#pragma unroll
-  for (int ax = 0; ax < 3; ++ax) {
-    if (g.periodic[ax]) {
-      const float k = rintf(d[ax].hi * g.invL[ax]);
-      if (k != 0.f) d[ax] = df_add(d[ax], dfl{-k * g.L[ax].hi, -k * g.L[ax].lo});
-    }
-  }
-  const dfl r2 = df_add(df_add(df_mul(d[0], d[0]), df_mul(d[1], d[1])), df_mul(d[2], d[2]));
-  return df_sqrt(r2);
-}
-
-// Wendland psi_{3,1} without its constant factor (it cancels in W / S):
-// (1 - q/2)^4 (2q + 1), zero for q >= 2
-__device__ __forceinline__ dfl wendland_w_df(dfl q) {
-  dfl t = df_add(dfl{1.f, 0.f}, dfl{-0.5f * q.hi, -0.5f * q.lo});
-  if (t.hi <= 0.f) return dfl{0.f, 0.f};
-  const dfl t2 = df_mul(t, t);
-  return df_mul(df_mul(t2, t2), df_add(dfl{1.f, 0.f}, dfl{2.f * q.hi, 2.f * q.lo}));
-}
-
-// truncated Gaussian (Sec. 5.2, radius 3h): e^{-q^2} from the double-float q,
-// the exponential in float64 once per pair (the set-up runs once per A(dt))
-__device__ __forceinline__ dfl gauss_e_df(dfl q) { return df_from_double(exp(-df_to_double(df_mul(q, q)))); }
-
-// the fluid coefficient's kernel factor: (2 - q)^3 (Wendland) or e^{-q^2} (Gaussian),
-// each without the constant of |f| (it is in R_b)
-__device__ __forceinline__ dfl fluid_kernel_df(dfl q, int gauss) {
-  if (gauss) return gauss_e_df(q);
-  dfl tq = df_add(dfl{2.f, 0.f}, df_neg(q));
-  if (tq.hi <= 0.f) tq = dfl{0.f, 0.f};
-  return df_mul(df_mul(tq, tq), tq);
-}
-
-// the Shepard weight w(q) without its constant: Wendland, or e^{-q^2} - e^{-9}
-__device__ __forceinline__ dfl shepard_w_df(dfl q, int gauss, double gauss_tail) {
-  if (gauss) return df_from_double(exp(-df_to_double(df_mul(q, q))) - gauss_tail);
-  return wendland_w_df(q);
 }
 
 __global__ void k_op_count(const uint8_t* __restrict__ type, const int32_t* __restrict__ cnt,
@@ -219,14 +161,13 @@ __global__ void k_op_fill(const float4* __restrict__ pos, const float* __restric
   }
 }
 
-// y = A v (or D^-1 A v) in float32, one warp per 32-row slice, one row per lane.
-template <bool JACOBI>
+// y = A v in float32, one warp per 32-row slice, one row per lane.
 __global__ void __launch_bounds__(kBlock) k_apply_f32(OpView op, const float4* __restrict__ v, float4* __restrict__ y) {
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t sl = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; sl < op.nslices; sl += nwarps) {
     float4 vb;
-    y[sl * kSlice + lane] = apply_row<8, false, JACOBI>(op, v, sl, lane, vb);
+    y[sl * kSlice + lane] = apply_row<8, false, false>(op, v, sl, lane, vb);
   }
 }
 
@@ -377,15 +318,9 @@ sph_status ensure_wpart(sph_neighbors* H, int grid, cudaStream_t st) {
   return SPH_OK;
 }
 
-sph_status ensure_operator(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st) {
-  if (!P || !(P->dt > 0.0) || !std::isfinite(P->dt) || (P->boundary != SPH_BC_DUMMY && P->boundary != SPH_BC_DYNAMIC) ||
-      (P->mean != SPH_MEAN_HARMONIC && P->mean != SPH_MEAN_ARITHMETIC)) {
-    set_error("viscous parameters: dt must be positive and finite, boundary/mean one of the enums");
-    return SPH_ERR_INVALID;
-  }
-  if (H->op_valid && H->op_params.dt == P->dt && H->op_params.boundary == P->boundary &&
-      H->op_params.mean == P->mean && H->op_mu_version == H->mu_version)
-    return SPH_OK;
+// SELL-32 with 32-bit rows: k_op_count, the slice offsets (synchronises), k_op_fill
+static sph_status fill_ih(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st) {
+  SPH_TRY(ensure_nbr(H, st));
   OpGeom g{};
   for (int ax = 0; ax < 3; ++ax) {
     g.L[ax] = H->grid.L[ax];
@@ -394,11 +329,7 @@ sph_status ensure_operator(sph_neighbors* H, const sph_visc_params* P, cudaStrea
   }
   g.h = (double)H->h;
   g.inv_h = 1.0 / g.h;
-  SPH_TRY(H->op_cnt.alloc(H->n_pad));
-  SPH_TRY(H->op_kind.alloc(H->n_pad));
   SPH_TRY(H->op_off.alloc(H->nslices + 1));
-  SPH_TRY(H->invD.alloc(H->n_pad));
-  SPH_TRY(H->D64.alloc(H->n_pad));
   const int grid = grid_for(H, H->n_pad);
   SPH_LAUNCH(k_op_count, grid, kBlock, 0, st)(H->type_s.p, H->cnt.p, H->slice_off.p, H->nbr.p, H->n, H->n_pad,
                                               P->boundary, H->op_cnt.p, H->op_kind.p);
@@ -420,22 +351,57 @@ sph_status ensure_operator(sph_neighbors* H, const sph_visc_params* P, cudaStrea
                                              P->dt, P->mean, gauss, kf, std::exp(-kGaussK * kGaussK), H->op_ih.p,
                                              H->op_lo.p, H->invD.p, H->D64.p);
   SPH_TRY_CUDA(cudaGetLastError());
+  return SPH_OK;
+}
+
+sph_status ensure_operator(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st, OpForm form) {
+  if (!P || !(P->dt > 0.0) || !std::isfinite(P->dt) || (P->boundary != SPH_BC_DUMMY && P->boundary != SPH_BC_DYNAMIC) ||
+      (P->mean != SPH_MEAN_HARMONIC && P->mean != SPH_MEAN_ARITHMETIC)) {
+    set_error("viscous parameters: dt must be positive and finite, boundary/mean one of the enums");
+    return SPH_ERR_INVALID;
+  }
+  const bool tile = form == OP_FAST && H->tile_ok;
+  const bool same = H->op_valid && H->op_params.dt == P->dt && H->op_params.boundary == P->boundary &&
+                    H->op_params.mean == P->mean && H->op_mu_version == H->mu_version;
+  if (same && (tile ? H->op_tile_valid : H->op_ih_valid)) return SPH_OK;
+  if (!same) {
+    H->op_valid = H->op_tile_valid = H->op_ih_valid = false;
+    ++H->op_version;
+  }
+  SPH_TRY(H->op_cnt.alloc(H->n_pad));
+  SPH_TRY(H->op_kind.alloc(H->n_pad));
+  SPH_TRY(H->invD.alloc(H->n_pad));
+  SPH_TRY(H->D64.alloc(H->n_pad));
+  if (tile) {
+    SPH_TRY(tile_fill(H, P, st));
+    H->op_tile_valid = true;
+  } else {
+    SPH_TRY(fill_ih(H, P, st));
+    H->op_ih_valid = true;
+  }
   H->op_valid = true;
   H->op_params = *P;
   H->op_mu_version = H->mu_version;
-  ++H->op_version;
   return SPH_OK;
 }
 
 void launch_residual_f64(const sph_neighbors* H, int grid, const double* x, const double* b, double* r,
                          double* partials, unsigned int* counter, double* res_out, cudaStream_t st) {
   SPH_LAUNCH(k_split_x, grid_for(H, H->n_pad), kBlock, 0, st)(x, H->n_pad, H->v_x2.p);
+  if (H->op_tile_valid) {
+    tile_residual(H, grid, H->v_x2.p, x, b, r, partials, counter, res_out, st);
+    return;
+  }
   SPH_LAUNCH(k_residual_df, grid, kBlock, 0, st)(op_view(H), H->op_lo.p, H->v_x2.p, x, b, r, H->n,
                                                  partials, counter, res_out);
 }
 
 void launch_residual_update(const sph_neighbors* H, int grid, const float4* d, double* r, double* partials,
                             unsigned int* counter, double* res_out, cudaStream_t st) {
+  if (H->op_tile_valid) {
+    tile_residual_update(H, grid, d, r, partials, counter, res_out, st);
+    return;
+  }
   SPH_LAUNCH(k_residual_update_df, grid, kBlock, 0, st)(op_view(H), H->op_lo.p, d, r, H->n, partials, counter,
                                                         res_out);
 }
@@ -448,11 +414,14 @@ OpView op_view(const sph_neighbors* H) {
                 wp ? H->wpart.p : nullptr, wp ? H->wpart_nw : 0};
 }
 
-void launch_apply_f32(const sph_neighbors* H, const float4* v, float4* y, bool jacobi, cudaStream_t st) {
+void launch_apply_f32(const sph_neighbors* H, const float4* v, float4* y, cudaStream_t st) {
+  if (H->op_tile_valid) {
+    tile_apply(H, v, y, false, st);
+    return;
+  }
   const int grid = grid_for(H, H->nslices * 32);
   const OpView op = op_view(H);
-  auto kern = jacobi ? k_apply_f32<true> : k_apply_f32<false>;
-  SPH_LAUNCH(kern, grid, kBlock, 0, st)(op, v, y);
+  SPH_LAUNCH(k_apply_f32, grid, kBlock, 0, st)(op, v, y);
 }
 
 sph_status visc_apply(sph_neighbors* H, const sph_visc_params* P, const float* v, float* y, cudaStream_t st) {
@@ -461,6 +430,17 @@ sph_status visc_apply(sph_neighbors* H, const sph_visc_params* P, const float* v
     return SPH_ERR_INVALID;
   }
   SPH_TRY(ensure_operator(H, P, st));
+  const uintptr_t v0 = reinterpret_cast<uintptr_t>(v), y0 = reinterpret_cast<uintptr_t>(y);
+  const uintptr_t len = (uintptr_t)H->n * sizeof(float4);
+  if (H->op_tile_valid && (v0 >= y0 + len || y0 >= v0 + len)) {
+    // the tile kernel reads v and writes y through perm: no sorted copies (the two
+    // copies below took 7 of 45 us on the 274k box)
+    standalone_begin(H, st);
+    tile_apply(H, reinterpret_cast<const float4*>(v), reinterpret_cast<float4*>(y), true, st);
+    SPH_TRY(standalone_end(H, st, 0));
+    SPH_TRY_CUDA(cudaGetLastError());
+    return SPH_OK;
+  }
   SPH_TRY(H->v_tmp.alloc(2 * H->n_pad));
   float4* vs = H->v_tmp.p;
   float4* ys = H->v_tmp.p + H->n_pad;
@@ -468,7 +448,7 @@ sph_status visc_apply(sph_neighbors* H, const sph_visc_params* P, const float* v
   SPH_LAUNCH(k_gather_f4, grid, kBlock, 0, st)(v, H->perm.p, H->n, H->n_pad, vs);
   SPH_TRY_CUDA(cudaGetLastError());
   standalone_begin(H, st);
-  launch_apply_f32(H, vs, ys, false, st);
+  launch_apply_f32(H, vs, ys, st);
   SPH_TRY(standalone_end(H, st, 0));
   SPH_TRY_CUDA(cudaGetLastError());
   SPH_LAUNCH(k_scatter_f4, grid, kBlock, 0, st)(ys, H->perm.p, H->n, y);

@@ -127,6 +127,7 @@ sph_status set_viscosity_impl(sph_neighbors* H, const float* mu, cudaStream_t st
 
 sph_status mu_papanastasiou(sph_neighbors* H, const float* vel, const float* wall_vel, double tau0, double mu0,
                             double m, float* mu_out, int set_handle, cudaStream_t st) {
+  SPH_TRY(ensure_nbr(H, st));
   MuGeom g{};
   for (int ax = 0; ax < 3; ++ax) {
     g.L[ax] = (float)H->grid.L[ax];

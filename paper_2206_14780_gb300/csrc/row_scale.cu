@@ -107,7 +107,7 @@ __global__ void k_rs_apply(const float* __restrict__ rs, const int32_t* __restri
 
 sph_status row_norms_impl(sph_neighbors* H, const sph_visc_params* P, int mode, double factor, double power,
                           float* out, cudaStream_t st) {
-  SPH_TRY(ensure_operator(H, P, st));
+  SPH_TRY(ensure_operator(H, P, st, OP_IH));
   SPH_LAUNCH(k_row_norms, grid_for(H, H->n), kBlock, 0, st)(H->op_off.p, H->op_cnt.p, H->op_ih.p, H->op_kind.p,
                                                              H->invD.p, H->perm.p, H->n, mode, (float)factor,
                                                              (float)power, out);
@@ -207,7 +207,7 @@ sph_status sph_mlp_scale_targets(sph_neighbors* h, const sph_visc_params* params
   }
   if (!scale_args_ok("sph_mlp_scale_targets", factor, power)) return SPH_ERR_INVALID;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  SPH_TRY(ensure_operator(h, params, st));
+  SPH_TRY(ensure_operator(h, params, st, OP_IH));
   SPH_LAUNCH(k_scale_targets, grid_for(h, h->n), kBlock, 0, st)(h->op_off.p, h->op_cnt.p, h->op_ih.p, h->op_kind.p,
                                                                  h->invD.p, h->type_s.p, h->perm.p, h->n,
                                                                  (float)std::log(factor), (float)power,

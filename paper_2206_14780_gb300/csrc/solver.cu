@@ -30,6 +30,7 @@
 // ||r64|| / ||b|| <= rtol, else run a pass on D^-1 r64, add d to x (float64)
 // and update r64 -= A d in double-float arithmetic; the residual that accepts
 // the solution is recomputed from x.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -38,6 +39,7 @@
 #include "bicgstab_scalars.cuh"
 #include "reduce.cuh"
 #include "sph_internal.cuh"
+#include "tiles.cuh"
 
 namespace sph {
 
@@ -436,6 +438,67 @@ __global__ void __launch_bounds__(kBlock, 3) k_apply_dot_union(OpView op, const 
   dots_finish<PH>(acc, S, partials, counter);
 }
 
+// The apply of the tile form (tiles.cuh): one block of 256 threads per tile, the
+// tile's distinct neighbour vectors copied once into shared memory (cp.async), then
+// 6 bytes of stream per entry (16-bit position, float32 coefficient) and one 16-byte
+// shared-memory gather.  The SELL-32 forms stream 8 bytes and gather through L1,
+// whose tag look-ups (one per distinct line, ~17 per warp and entry) set their pace.
+// In the solve loop of the 1.16M box: 137 us -> 128 / 124 us per apply (A p / A r*);
+// alone (sph_visc_apply): 144 -> 109 us for ~600 MB, 88% of the measured copy
+// bandwidth with the gathers left out and 81% with them, so what is left in the loop
+// is the reduction at the end and the launch.  2 groups of 4 entries in flight per
+// lane and 5 blocks per SM measured best of 1-4 groups and 3-6 blocks; an L2 prefetch of the
+// stream (bulk, 6-16 groups ahead) made it slower (141-163 us).
+template <int PH, int TS>
+__global__ void __launch_bounds__(256, kTileBlocks) k_tile_apply_dot(TileView op, const float4* __restrict__ v,
+                                                        float4* __restrict__ y, const float4* __restrict__ rh,
+                                                        SolverScalars* S, double* partials, unsigned int* counter) {
+  constexpr int K = PhaseDots<PH>::K, SP = 8 / TS, R = 32 * TS;
+  extern __shared__ __align__(16) float4 u[];
+  __shared__ float part[SP > 1 ? (SP - 1) * R * 3 : 1];
+  griddep_wait();
+  if (S->done) return;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int split = wid / TS, row = (wid % TS) * 32 + lane;
+  float acc[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) acc[k] = 0.f;
+  for (int64_t tile = blockIdx.x; tile < op.ntiles; tile += gridDim.x) {
+    tile_load_union(op, tile, v, u);
+    const int64_t sl = tile * TS + wid % TS, s = sl * kSlice + lane;
+    const bool have = sl < op.nslices;
+    int c = 0;
+    uint8_t kd = KIND_IDENTITY;
+    float4 vb = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (have) {
+      c = op.cnt[s];
+      kd = op.kind[s];
+      vb = v[s];
+    }
+    const float kap = kd == KIND_FLUID ? 1.f : 0.f;
+    TileStream ts;
+    ts.start(op, sl, lane, c, split, SP);
+    cp_async_wait_all();
+    __syncthreads();
+    float ax = 0.f, ay = 0.f, az = 0.f;
+    ts.sum(u, split, SP, kap * vb.x, kap * vb.y, kap * vb.z, ax, ay, az);
+    tile_combine<TS>(part, split, row, ax, ay, az);
+    if (have && split == 0) {
+      const float4 o = tile_finish(kd, vb, ax, ay, az, PH != PH_CG ? op.invD[s] : 1.f);
+      y[s] = o;
+      dots_row<PH>(acc, o, vb, rh, s);
+    }
+    __syncthreads();
+  }
+  dots_finish<PH>(acc, S, partials, counter);
+}
+
+using TileDotFn = void (*)(TileView, const float4*, float4*, const float4*, SolverScalars*, double*, unsigned int*);
+template <int PH>
+TileDotFn tile_dot_kernel(int ts) {
+  return ts == 8 ? k_tile_apply_dot<PH, 8> : (ts == 4 ? k_tile_apply_dot<PH, 4> : k_tile_apply_dot<PH, 2>);
+}
+
 }  // namespace
 
 // [phase][variant] with variants (U, PF) = (8,0), (4,0), (8,1), (4,1) as in apply.cuh,
@@ -744,7 +807,8 @@ sph_status ensure_workspace(sph_neighbors* H) {
       }
     H->red_grid = H->num_sms * best;
   }
-  SPH_TRY(H->partials.alloc((size_t)H->red_grid * kMaxDots));
+  H->red_cap = std::max(H->red_grid, 8 * H->num_sms);
+  SPH_TRY(H->partials.alloc((size_t)H->red_cap * kMaxDots));
   if (!H->counters.p) {
     SPH_TRY(H->counters.alloc(CNT_COUNT));
     SPH_TRY_CUDA(cudaMemset(H->counters.p, 0, CNT_COUNT * sizeof(unsigned int)));
@@ -793,10 +857,25 @@ static cudaError_t loop_launch(bool pdl, void (*kernel)(KArgs...), int grid, siz
   return cudaGetLastError();
 }
 
+// the tile form of a solve's applies: which view, and the grid per phase
+struct TileApply {
+  bool on = false;
+  TileView view{};
+  size_t smem = 0;
+  int grid[4] = {0, 0, 0, 0};
+};
+
 template <int PH>
-static cudaError_t launch_apply_dot(sph_neighbors* H, bool pdl, int grid, const OpView& op, const float4* v,
-                                    float4* y, const float4* rh, SolverScalars* S, unsigned int* counter,
-                                    cudaStream_t st) {
+static cudaError_t launch_apply_dot(sph_neighbors* H, bool pdl, int grid, const OpView& op, const TileApply& T,
+                                    const float4* v, float4* y, const float4* rh, SolverScalars* S,
+                                    unsigned int* counter, cudaStream_t st) {
+  if (T.on) {
+    prof_begin(H, st, PH == PH_DELTA ? 0 : 1);
+    const TileDotFn kern = tile_dot_kernel<PH>(H->tile_ts);
+    const cudaError_t e = loop_launch(pdl, kern, T.grid[PH], T.smem, st, T.view, v, y, rh, S, H->partials.p, counter);
+    prof_end(H, st);
+    return e;
+  }
   const bool forced = H->force_form >= 0;
   // the CG phase runs the register form the tuner chose for the delta phase (same dots)
   const int tp = PH == PH_CG ? PH_DELTA : PH;
@@ -818,15 +897,25 @@ sph_status solve_mixed(sph_neighbors* H, const sph_visc_params* P, const sph_sol
                        double* x, sph_solve_report* R, cudaStream_t st) {
   SPH_TRY(ensure_operator(H, P, st));
   SPH_TRY(ensure_workspace(H));
-  // balanced slice ranges for the grid of the float64 residual kernels
-  SPH_TRY(ensure_wpart(H, red_grid_for(H, H->n_pad), st));
-  SPH_TRY(autotune_apply(H, O->merged_reductions != 0, H->counters.p + CNT_TUNE, st));
+  // The tile form where the operator has it.  It is faster than every form below at
+  // every size measured (see k_tile_apply_dot), so nothing is timed for it; a forced
+  // apply_form, and particle sets without tiles, take the SELL-32 forms.
+  TileApply T;
+  T.on = H->op_tile_valid && O->apply_form == 0;
+  if (!T.on) {
+    SPH_TRY(ensure_operator(H, P, st, OP_IH));
+    // balanced slice ranges for the grid of the float64 residual kernels
+    SPH_TRY(ensure_wpart(H, red_grid_for(H, H->n_pad), st));
+    SPH_TRY(autotune_apply(H, O->merged_reductions != 0, H->counters.p + CNT_TUNE, st));
+  }
   const int64_t np = H->n_pad;
   const int grid_rows = red_grid_for(H, np);
   const int grid_slices = red_grid_for(H, H->nslices * 32);
   // the chosen forms' prerequisites (the unions of form 5 follow the operator)
-  SPH_TRY(apply_prepare(H, H->apply_var[PH_DELTA], st));
-  SPH_TRY(apply_prepare(H, H->apply_var[O->merged_reductions ? PH_OMEGA_MERGED : PH_OMEGA], st));
+  if (!T.on) {
+    SPH_TRY(apply_prepare(H, H->apply_var[PH_DELTA], st));
+    SPH_TRY(apply_prepare(H, H->apply_var[O->merged_reductions ? PH_OMEGA_MERGED : PH_OMEGA], st));
+  }
   H->force_form = -1;
   if (O->launch_mode < 0 || O->launch_mode > 1) {
     set_error("sph_visc_solve: launch_mode %d is neither 0 nor 1", O->launch_mode);
@@ -873,6 +962,18 @@ sph_status solve_mixed(sph_neighbors* H, const sph_visc_params* P, const sph_sol
   OpView op = op_view(H);
   if (H->row_scaled) op.invD = H->invD_sc.p;
   const float* invD = op.invD;
+  if (T.on) {
+    T.view = tile_view(H);
+    T.view.invD = invD;
+    T.smem = tile_smem(H, 16);
+    const TileDotFn k[4] = {tile_dot_kernel<PH_DELTA>(H->tile_ts), tile_dot_kernel<PH_OMEGA>(H->tile_ts),
+                            tile_dot_kernel<PH_OMEGA_MERGED>(H->tile_ts), tile_dot_kernel<PH_CG>(H->tile_ts)};
+    for (int ph = 0; ph < 4; ++ph) {
+      T.grid[ph] = tile_grid(H, (const void*)k[ph], T.smem);
+      T.grid[ph] = std::min(T.grid[ph], H->red_cap);   // the partials are sized for it
+    }
+  }
+  H->tile_grid = T.on ? T.grid[cg ? PH_CG : PH_DELTA] : 0;
   const double* D64 = H->row_scaled ? H->D64_sc.p : H->D64.p;
   SolverScalars* S = H->scal.p;
   unsigned int* C = H->counters.p;
@@ -979,18 +1080,18 @@ sph_status solve_mixed(sph_neighbors* H, const sph_visc_params* P, const sph_sol
       for (int it = 0; it < chunk; ++it) {
         if (cg) {
           keep(loop_launch(pdl, k_cg_p, grid_rows, 0, st, np, V, invD, jacobi, S));
-          keep(launch_apply_dot<PH_CG>(H, pdl, grid_slices, op, V.p, V.Ap, V.rh, S, C + CNT_CG_A, st));
+          keep(launch_apply_dot<PH_CG>(H, pdl, grid_slices, op, T, V.p, V.Ap, V.rh, S, C + CNT_CG_A, st));
           keep(loop_launch(pdl, k_cg_xr, grid_rows, 0, st, np, V, invD, jacobi, S, H->partials.p, C + CNT_CG_XR));
           continue;
         }
         if (!merged) keep(loop_launch(pdl, k_p_update, grid_rows, 0, st, np, V, S));
-        keep(launch_apply_dot<PH_DELTA>(H, pdl, grid_slices, op, V.p, V.Ap, V.rh, S, C + CNT_DELTA, st));
+        keep(launch_apply_dot<PH_DELTA>(H, pdl, grid_slices, op, T, V.p, V.Ap, V.rh, S, C + CNT_DELTA, st));
         keep(loop_launch(pdl, k_rstar, grid_rows, 0, st, np, V, S));
         if (merged) {
-          keep(launch_apply_dot<PH_OMEGA_MERGED>(H, pdl, grid_slices, op, V.rs, V.As, V.rh, S, C + CNT_OMEGA, st));
+          keep(launch_apply_dot<PH_OMEGA_MERGED>(H, pdl, grid_slices, op, T, V.rs, V.As, V.rh, S, C + CNT_OMEGA, st));
           keep(loop_launch(pdl, k_xrp_update, grid_rows, 0, st, np, V, S, C + CNT_XRP));
         } else {
-          keep(launch_apply_dot<PH_OMEGA>(H, pdl, grid_slices, op, V.rs, V.As, V.rh, S, C + CNT_OMEGA, st));
+          keep(launch_apply_dot<PH_OMEGA>(H, pdl, grid_slices, op, T, V.rs, V.As, V.rh, S, C + CNT_OMEGA, st));
           keep(loop_launch(pdl, k_xr_update, grid_rows, 0, st, np, V, S, H->partials.p, C + CNT_XR));
         }
       }

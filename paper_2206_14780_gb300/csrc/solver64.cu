@@ -259,7 +259,7 @@ enum { C64_INIT = 0, C64_DELTA, C64_OMEGA, C64_XR, C64_RES, C64_NORM, C64_COUNT 
 
 sph_status solve_fp64(sph_neighbors* H, const sph_visc_params* P, const sph_solve_opts* O, const double* b, double* x,
                       sph_solve_report* R, cudaStream_t st) {
-  SPH_TRY(ensure_operator(H, P, st));
+  SPH_TRY(ensure_operator(H, P, st, OP_IH));
   SPH_TRY(ensure_workspace(H));
   const int64_t np = H->n_pad;
   for (int k = 0; k < 6; ++k) SPH_TRY(H->w64[k].alloc(3 * np));

@@ -194,8 +194,28 @@ struct sph_neighbors {
   int64_t nnz = 0, nnz_pad = 0;
   int32_t max_cnt = 0;
 
-  // operator (coefficients of A(dt)) SELL-32
-  bool op_valid = false;
+  // The lists above are kept as 16-bit positions per tile (tiles.cuh) where the
+  // particle set allows it (tile_ok); nbr and slice_off are then made on demand
+  // (ensure_nbr) for the kernels that walk 32-bit rows.
+  int32_t maxnb = 0;               // capacity of the lists
+  bool tile_ok = false, nbr_valid = false;
+  int tile_ts = 8;                 // slices per tile
+  int64_t ntiles = 0, t_istride = 0, t_entries = 0;
+  int32_t t_ustride = 0, tile_umax = 0;
+  sph::DBuf<uint16_t> t_idx;       // [nslices][t_istride] union positions x 16
+  sph::DBuf<uint16_t> t_raw;       // [n_pad max_neighbors] places in the tile's search region (scratch)
+  sph::DBuf<int2> t_cells;         // [ntiles][kTileCells + 1] (first row, region offset) of the region's cells
+  sph::DBuf<int32_t> t_ncell, t_unum, t_uni;   // cells per region, union sizes, unions [ntiles][t_ustride]
+  sph::DBuf<int32_t> t_nfl;        // [n_pad] interleaved entries (fluid rows: all; wall rows: the fluid ones)
+  sph::DBuf<int64_t> t_off;        // [nslices + 1] entry offsets of t_hi, t_lo
+  sph::DBuf<float> t_hi, t_lo;     // the operator's coefficients in the order of t_idx
+  sph::DBuf<unsigned long long> t_nnz;   // coefficients of the tile form (op_nnz when that is -1)
+  sph::DBuf<int32_t> tmp_ids;      // particles by cell, unordered
+  sph::DBuf<long long> scan_sums;  // tile sums of a scan
+
+  // operator (coefficients of A(dt)): valid in the tile form, in SELL-32 with
+  // 32-bit rows, or both, for the parameters op_params
+  bool op_valid = false, op_tile_valid = false, op_ih_valid = false;
   sph_visc_params op_params{};
   uint64_t mu_version = 0, op_mu_version = ~0ull;
   sph::DBuf<int32_t> op_cnt;       // [n_pad]
@@ -242,7 +262,8 @@ struct sph_neighbors {
   sph::DBuf<sph::SolverScalars> scal;
   int32_t* host_flags = nullptr;     // pinned [4]
   sph::SolverScalars* host_scal = nullptr;  // pinned
-  int red_grid = 0;                  // blocks of the reducing kernels
+  int red_grid = 0;                  // blocks of the reducing row kernels
+  int red_cap = 0;                   // most blocks any reducing kernel has
   // apply autotuner (autotune.cu): chosen row-loop form and grid per phase
   int apply_var[3] = {0, 0, 0};
   int apply_grid[3] = {0, 0, 0};
@@ -258,6 +279,7 @@ struct sph_neighbors {
   double pass_dt[2] = {-1.0, -1.0};
   int pass_slot_next = 0;
   int force_grid = 0;
+  int tile_grid = 0;                 // blocks of the tile apply in the last mixed solve, 0: another form
   sph::DBuf<sph::SolverScalars> scal_tune;
 
   // instrumentation (sph_profile_*)
@@ -302,9 +324,8 @@ struct sph_neighbors {
 namespace sph {
 
 // neighbors.cu
-sph_status scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t m, cudaStream_t st);
-sph_status slice_offsets(const int32_t* cnt, int64_t nslices, int64_t* off, int32_t* width_tmp,
-                         cudaStream_t st);
+// the 32-bit rows of the lists (nbr, slice_off), expanded from the tiles if need be
+sph_status ensure_nbr(sph_neighbors* H, cudaStream_t st);
 
 sph_status build_slices(sph_neighbors* H, const int32_t* cnt, int64_t* off, int64_t* total_pad, int64_t* total,
                         int32_t* maxc, cudaStream_t st);
@@ -323,8 +344,19 @@ sph_status ensure_wpart(sph_neighbors* H, int grid, cudaStream_t st);
 sph_status visc_apply(sph_neighbors* H, const sph_visc_params* P, const float* v, float* y, cudaStream_t st);
 sph_status visc_apply_noalloc(sph_neighbors* H, const sph_visc_params* P, const float* v, float* y,
                               cudaStream_t st);
-sph_status ensure_operator(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st);
-void launch_apply_f32(const sph_neighbors* H, const float4* v, float4* y, bool jacobi, cudaStream_t st);
+// A(dt) on the handle: the tile form where the lists have one, else SELL-32 with
+// 32-bit rows; OP_IH asks for the latter whatever the lists are
+enum OpForm { OP_FAST, OP_IH };
+sph_status ensure_operator(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st, OpForm form = OP_FAST);
+// tiles.cu: coefficients in the tile form; y = A v and the residuals with them
+sph_status tile_fill(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st);
+void tile_apply(const sph_neighbors* H, const float4* v, float4* y, bool caller_order, cudaStream_t st);
+void tile_wall_close(const sph_neighbors* H, double* x0, const double* b, cudaStream_t st);
+void tile_residual(const sph_neighbors* H, int grid, const float4* x2, const double* x, const double* b, double* r,
+                   double* partials, unsigned int* counter, double* res_out, cudaStream_t st);
+void tile_residual_update(const sph_neighbors* H, int grid, const float4* d, double* r, double* partials,
+                          unsigned int* counter, double* res_out, cudaStream_t st);
+void launch_apply_f32(const sph_neighbors* H, const float4* v, float4* y, cudaStream_t st);
 // apply_otf.cu: y = A v with the coefficients recomputed per pair
 void launch_apply_otf(const sph_neighbors* H, const float4* v, float4* y, bool jacobi, cudaStream_t st);
 // apply_union.cu: per-slice unions for apply form 5 (built once per operator)

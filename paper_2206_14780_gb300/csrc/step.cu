@@ -311,6 +311,7 @@ sph_status evaluate(sph_state* S, const sph_step_params* Pp, sph_neighbors** han
   SPH_TRY(T.P_s.alloc(H->n_pad));
   if (Pp->rheology == 1)
     SPH_TRY(mu_papanastasiou(H, S->vel, S->vel, Pp->tau0, Pp->mu0, Pp->m, S->mu, 1, st));
+  SPH_TRY(ensure_nbr(H, st));
   const StepGeom g = step_geom(H, S);
   const int grid = grid_for(H, H->n);
   SPH_LAUNCH(k_step_eos, grid, kBlock, 0, st)(H->rho_s.p, H->n, Pp->rho0, Pp->c0, Pp->zeta, T.P_s.p);
