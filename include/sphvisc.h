@@ -246,7 +246,10 @@ typedef struct {
   int32_t launch_mode;     /* 0: the BiCGSTAB loop's kernels are programmatic
                               dependent launches, each launch processed while its
                               predecessor still runs (default); 1: plain
-                              stream-ordered launches.  Same results either way   */
+                              stream-ordered launches.  Same results either way;
+                              sets of up to about 100k particles run as one
+                              cooperative kernel under both (BiCGSTAB, direct
+                              reductions, apply_form 0, profiling off)            */
   int32_t method;          /* SPH_SOLVER_BICGSTAB (default) or SPH_SOLVER_CG      */
 } sph_solve_opts;
 

@@ -676,7 +676,7 @@ struct Fields<true> {
 // region's particles that some row references are marked, the marks are turned
 // into positions by ballots and a prefix sum, and one thread per row sorts its
 // entries into the 8 bank groups (position mod 8) and takes them out again so that
-// lane l takes group (l + j - 1) mod 8 at step j while that group lasts, then the
+// lane l takes group (l + j - 2) mod 8 at step j while that group lasts, then the
 // fullest one.  Wall rows: fluid neighbours first, then, at the next multiple of
 // four entries, the wall neighbours; nfl counts the former.
 template <int TS, bool WIDE>
@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(256) k_tile_plan(const uint8_t* __restrict__ t
     for (int k = 0; k < 4; ++k) {
       v[k] = fill;
       if (j0 + k < nf) {
-        int b = (rl + k + j0 + 7) & 7;
+        int b = (rl + k + j0 + 6) & 7;
         if (left.get(b) == 0) {
           int most = 0;
 #pragma unroll
@@ -972,21 +972,25 @@ sph_status build_slices(sph_neighbors* H, const int32_t* cnt, int64_t* off, int6
 }
 
 // places in shared memory for a tile's search region; 256-row tiles of the box need
-// up to ~3,100 (2,757 particles and the cells' padding), the Gaussian's 128-row tiles
-// 2,304, h = 2.5 dp 6,656
-constexpr int kRegionSmall = 3584;
+// up to ~3,100 (2,757 particles and the cells' padding), the Gaussian's narrow channels
+// ~3,600, h = 2.5 dp 6,656
+constexpr int kRegionSmall = 4608;
 constexpr int kRegionLarge = 7168;
 
 // Slices per tile.  Large tiles share more of their neighbours (4.4 union rows per row
 // at 8 slices, 5.8 at 4, 7.8 at 2 on the box); small ones give a small set more blocks
-// and a row more threads.  Apply in the solve loop, us at 8 / 4 / 2 slices: 15.6k rows
-// 14.7 / 12.6 / 12.5, 27k 14.6 / 13.5 / 12.9, 64k 17.3 / 16.5 / 18.0, 274k 37.5 / 37.5 /
-// 41.4, 1,157k 128 / 138 / 161.  The Gaussian's unions are larger and its rows longer:
-// 26k rows 25 / 20.8 / 17.4, 77k 36.4 / 28.6 / 30.6, 190k 67.8 / 53.6 / 56.4.  Beyond 640
-// entries per row the lists of 4 slices exceed the plan's shared memory.
-static int tile_slices_for(int64_t nslices, int32_t maxnb) {
-  if (nslices < 1100 || maxnb > 640) return 2;
-  return maxnb > 160 ? 4 : 8;
+// and a row more threads.  Whole solves at 8 / 4 / 2 slices in the cooperative kernel
+// (persist.cu): 2.2k rows 837 / 761 / 810 us, 6.8k 1476 / 1392 / 1465, 16k 1865 / 1981 /
+// 2059, 30k 2609 / 2690 / 3162, 51k 3790 / 3543 / 3747; only 8 slices fit at 104k.  Applies of the
+// five-kernel loop: 64k rows 17.3 / 16.5 / 18.0 us, 274k 37.5 / 37.5 / 41.4, 1,157k 128 / 138 / 161.
+// The Gaussian's unions are larger and its rows longer: apply at 190k rows 67.8 / 53.6 /
+// 56.4, but at 77k the cooperative kernel holds 8 slices better (6117 / 7213 us a solve).
+// Beyond 320 (640) entries per row the lists of 8 (4) slices exceed the plan's shared
+// memory.
+static int tile_slices_for(int64_t nslices, int32_t maxnb, int num_sms) {
+  if (nslices < 600 || maxnb > 640) return 2;
+  if (nslices < 1800 || maxnb > 320) return 4;
+  return maxnb > 160 && nslices > 18 * (int64_t)num_sms ? 4 : 8;
 }
 
 static sph_status fixed_offsets(sph_neighbors* H, cudaStream_t st) {
@@ -1033,7 +1037,7 @@ static sph_status launch_search_ts(sph_neighbors* H, const Grid& g, const BandIn
 // search and plan of every tile, and the coefficient offsets of the slices
 static sph_status launch_tile_search(sph_neighbors* H, const Grid& g, const BandIn& bin, int32_t maxnb, int cap,
                                      cudaStream_t st) {
-  const int ts = tile_slices_for(H->nslices, maxnb);
+  const int ts = tile_slices_for(H->nslices, maxnb, H->num_sms);
   H->tile_ts = ts;
   H->ntiles = (H->nslices + ts - 1) / ts;
   H->t_istride = 32 * (((maxnb + 3) & ~3) + 4);

@@ -389,7 +389,7 @@ void launch_residual_f64(const sph_neighbors* H, int grid, const double* x, cons
                          double* partials, unsigned int* counter, double* res_out, cudaStream_t st) {
   SPH_LAUNCH(k_split_x, grid_for(H, H->n_pad), kBlock, 0, st)(x, H->n_pad, H->v_x2.p);
   if (H->op_tile_valid) {
-    tile_residual(H, grid, H->v_x2.p, x, b, r, partials, counter, res_out, st);
+    tile_residual(H, H->v_x2.p, x, b, r, partials, counter, res_out, st);
     return;
   }
   SPH_LAUNCH(k_residual_df, grid, kBlock, 0, st)(op_view(H), H->op_lo.p, H->v_x2.p, x, b, r, H->n,
@@ -399,7 +399,7 @@ void launch_residual_f64(const sph_neighbors* H, int grid, const double* x, cons
 void launch_residual_update(const sph_neighbors* H, int grid, const float4* d, double* r, double* partials,
                             unsigned int* counter, double* res_out, cudaStream_t st) {
   if (H->op_tile_valid) {
-    tile_residual_update(H, grid, d, r, partials, counter, res_out, st);
+    tile_residual_update(H, d, r, partials, counter, res_out, st);
     return;
   }
   SPH_LAUNCH(k_residual_update_df, grid, kBlock, 0, st)(op_view(H), H->op_lo.p, d, r, H->n, partials, counter,

@@ -39,6 +39,7 @@
 #include "bicgstab_scalars.cuh"
 #include "reduce.cuh"
 #include "sph_internal.cuh"
+#include "persist.cuh"
 #include "tiles.cuh"
 
 namespace sph {
@@ -1000,6 +1001,11 @@ sph_status solve_mixed(sph_neighbors* H, const sph_visc_params* P, const sph_sol
   const int jacobi = O->jacobi ? 1 : 0;
   const bool pdl = O->launch_mode == 0;
 
+  // the cooperative kernel where the tiles are all resident at once; profiling times
+  // the applies as launches of their own
+  PersistPlan persist;
+  if (T.on && !cg && !merged && !H->prof_on) persist = persist_plan(H);
+
   std::memset(R, 0, sizeof(*R));
   int total_iters = 0, passes = 0;
   // Launch chunks: the host checks the device's stop flag after each chunk, and
@@ -1053,6 +1059,29 @@ sph_status solve_mixed(sph_neighbors* H, const sph_visc_params* P, const sph_sol
       break;
     }
     if (ref >= max_ref || total_iters >= maxit) break;
+    if (persist.ok) {
+      PersistResult pr;
+      SPH_TRY(persist_solve(H, persist, T.view, D64, rtol * bnorm, eps_floor, rr, maxit - total_iters, max_ref - ref, &pr,
+                            st));
+      passes += pr.passes;
+      ref += pr.passes - 1;   // the loop counts one
+      total_iters += pr.iters;
+      for (int c = 0; c < 3; ++c) {
+        R->state[c] = (int8_t)pr.state[c];
+        R->stalled_any[c] |= (int8_t)((pr.stalled >> c) & 1);
+        rr[c] = pr.rr[c];
+      }
+      if (pr.stuck) {
+        SPH_TRY(true_residual(H, st, rr));
+        rr_full = true;
+        const double rnorm2 = std::sqrt(rr[0] + rr[1] + rr[2]);
+        status = rnorm2 <= rtol * bnorm ? SPH_OK : SPH_NOT_CONVERGED;
+        break;
+      }
+      have_rr = true;
+      rr_full = false;
+      continue;
+    }
     // inner pass: ask it for what the outer loop still needs (with a 4x margin),
     // but never for more than eps_floor (float32 recursions stall below that)
     const double eps = std::fmax(eps_floor, 0.25 * rtol * bnorm / rnorm);

@@ -279,6 +279,8 @@ struct sph_neighbors {
   double pass_dt[2] = {-1.0, -1.0};
   int pass_slot_next = 0;
   int force_grid = 0;
+  sph::DBuf<double> persist_buf;     // block partials, result and barrier of the cooperative solve
+  void* host_persist = nullptr;      // pinned copy of its result
   int tile_grid = 0;                 // blocks of the tile apply in the last mixed solve, 0: another form
   sph::DBuf<sph::SolverScalars> scal_tune;
 
@@ -352,9 +354,9 @@ sph_status ensure_operator(sph_neighbors* H, const sph_visc_params* P, cudaStrea
 sph_status tile_fill(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st);
 void tile_apply(const sph_neighbors* H, const float4* v, float4* y, bool caller_order, cudaStream_t st);
 void tile_wall_close(const sph_neighbors* H, double* x0, const double* b, cudaStream_t st);
-void tile_residual(const sph_neighbors* H, int grid, const float4* x2, const double* x, const double* b, double* r,
+void tile_residual(const sph_neighbors* H, const float4* x2, const double* x, const double* b, double* r,
                    double* partials, unsigned int* counter, double* res_out, cudaStream_t st);
-void tile_residual_update(const sph_neighbors* H, int grid, const float4* d, double* r, double* partials,
+void tile_residual_update(const sph_neighbors* H, const float4* d, double* r, double* partials,
                           unsigned int* counter, double* res_out, cudaStream_t st);
 void launch_apply_f32(const sph_neighbors* H, const float4* v, float4* y, cudaStream_t st);
 // apply_otf.cu: y = A v with the coefficients recomputed per pair

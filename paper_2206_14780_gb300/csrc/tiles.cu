@@ -294,50 +294,6 @@ __global__ void __launch_bounds__(256) k_tile_wall_close(TileView op, const uint
   }
 }
 
-// A row's operator sum in double-float arithmetic over the tile form (residual_row
-// of residual_row.cuh with the gathers from shared memory).  X2: x = hi + lo in two
-// arrays uh, ul; else a float32 vector in uh.
-template <bool X2>
-__device__ __forceinline__ void tile_residual_row(const TileView& op, const float4* uh, const float4* ul, int64_t sl,
-                                                  int lane, int c, int first, int step, float4 kh, float4 kl,
-                                                  DFAcc& a0, DFAcc& a1, DFAcc& a2) {
-  const int64_t o0 = op.off[sl];
-  const float4* __restrict__ ph = reinterpret_cast<const float4*>(op.hi + o0) + lane;
-  const float4* __restrict__ pl = reinterpret_cast<const float4*>(op.lo + o0) + lane;
-  const uint2* __restrict__ pi = reinterpret_cast<const uint2*>(op.idx + sl * op.istride) + lane;
-  const int ng = (c + 3) >> 2;
-  float4 h = make_float4(0.f, 0.f, 0.f, 0.f), l = h;
-  uint2 p = make_uint2(0u, 0u);
-  if (first < ng) {
-    h = __ldcs(ph + first * 32);
-    l = __ldcs(pl + first * 32);
-    p = __ldcs(pi + first * 32);
-  }
-  for (int g = first; g < ng; g += step) {
-    float4 hn = h, ln = l;
-    uint2 pn = p;
-    if (g + step < ng) {
-      hn = __ldcs(ph + (g + step) * 32);
-      ln = __ldcs(pl + (g + step) * 32);
-      pn = __ldcs(pi + (g + step) * 32);
-    }
-    uint32_t o[4];
-    tile_unpack(p, o);
-    const float hv[4] = {h.x, h.y, h.z, h.w}, lv[4] = {l.x, l.y, l.z, l.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float4 xh = tile_at(uh, o[k]);
-      const float4 xl = X2 ? tile_at(ul, o[k]) : make_float4(0.f, 0.f, 0.f, 0.f);
-      a0.add(hv[k], lv[k], kh.x, xh.x, kl.x, xl.x);
-      a1.add(hv[k], lv[k], kh.y, xh.y, kl.y, xl.y);
-      a2.add(hv[k], lv[k], kh.z, xh.z, kl.z, xl.z);
-    }
-    h = hn;
-    l = ln;
-    p = pn;
-  }
-}
-
 // X2: r = b - A x on sorted [n_pad][3] arrays, x2 = x in float32 halves (hi, lo
 // interleaved); else r -= A d.  Partial sums of r_c^2 go through the grid reduction
 // into res_out.  The gathers come from shared memory (32 or 16 bytes a union row),
@@ -500,20 +456,20 @@ void tile_wall_close(const sph_neighbors* H, double* x0, const double* b, cudaSt
   SPH_LAUNCH(kern, tile_grid(H, (const void*)kern, smem), 256, smem, st)(tile_view(H), H->type_s.p, H->perm.p, H->n, b, x0);
 }
 
-void tile_residual(const sph_neighbors* H, int grid, const float4* x2, const double* x, const double* b, double* r,
+void tile_residual(const sph_neighbors* H, const float4* x2, const double* x, const double* b, double* r,
                    double* partials, unsigned int* counter, double* res_out, cudaStream_t st) {
   auto kern = SPH_TILE_PICK(H, k_tile_residual, SPH_COMMA true);
   const size_t smem = tile_smem(H, 32);
-  const int g = tile_grid(H, (const void*)kern, smem);
-  SPH_LAUNCH(kern, g < grid ? g : grid, 256, smem, st)(tile_view(H), x2, x, b, r, H->n, partials, counter, res_out);
+  const int g = tile_grid(H, (const void*)kern, smem);   // partials hold red_cap blocks
+  SPH_LAUNCH(kern, g < H->red_cap ? g : H->red_cap, 256, smem, st)(tile_view(H), x2, x, b, r, H->n, partials, counter, res_out);
 }
 
-void tile_residual_update(const sph_neighbors* H, int grid, const float4* d, double* r, double* partials,
+void tile_residual_update(const sph_neighbors* H, const float4* d, double* r, double* partials,
                           unsigned int* counter, double* res_out, cudaStream_t st) {
   auto kern = SPH_TILE_PICK(H, k_tile_residual, SPH_COMMA false);
   const size_t smem = tile_smem(H, 16);
-  const int g = tile_grid(H, (const void*)kern, smem);
-  SPH_LAUNCH(kern, g < grid ? g : grid, 256, smem, st)(tile_view(H), d, nullptr, nullptr, r, H->n, partials, counter,
+  const int g = tile_grid(H, (const void*)kern, smem);   // partials hold red_cap blocks
+  SPH_LAUNCH(kern, g < H->red_cap ? g : H->red_cap, 256, smem, st)(tile_view(H), d, nullptr, nullptr, r, H->n, partials, counter,
                                                        res_out);
 }
 

@@ -8,7 +8,7 @@
 // ~1,150 distinct neighbours (18 KB as float4).  A gather from L1 costs one tag
 // look-up per distinct 128-byte line, ~17 per warp; a 16-byte gather from shared
 // memory costs one cycle per 8-lane quarter plus bank conflicts.  Each row's
-// entries are ordered so that lane l of a warp reads bank group (l + j - 1) mod 8 at
+// entries are ordered so that lane l of a warp reads bank group (l + j - 2) mod 8 at
 // step j while it has such an entry left (5.1 cycles per warp instead of 9.3 in
 // ascending order, counted on the host for the box).
 //
@@ -21,6 +21,7 @@
 #pragma once
 
 #include "apply.cuh"
+#include "dfloat.cuh"
 #include "sph_internal.cuh"
 
 namespace sph {
@@ -81,9 +82,10 @@ __device__ __forceinline__ const float4& tile_at(const float4* u, uint32_t off) 
 constexpr int kTileDepth = 2;
 constexpr int kTileBlocks = 5;   // resident blocks per SM asked of the compiler
 
-struct TileStream {
-  float4 a[kTileDepth];
-  uint2 p[kTileDepth];
+template <int D>
+struct TileStreamD {
+  float4 a[D];
+  uint2 p[D];
   const float4* ph;
   const uint2* pi;
   int ng, ngw;   // groups of this row, most groups of the warp's rows
@@ -97,26 +99,29 @@ struct TileStream {
     }
   }
   __device__ __forceinline__ void start(const TileView& op, int64_t sl, int lane, int c, int first, int step) {
+    start_at(op, sl, __any_sync(0xffffffffu, c > 0) ? op.off[sl] : 0, lane, c, first, step);
+  }
+  // o0 = op.off[sl]
+  __device__ __forceinline__ void start_at(const TileView& op, int64_t sl, int64_t o0, int lane, int c, int first,
+                                           int step) {
     ng = (c + 3) >> 2;
     ngw = __reduce_max_sync(0xffffffffu, ng);
-    if (ngw > 0) {
-      ph = reinterpret_cast<const float4*>(op.hi + op.off[sl]) + lane;
-      pi = reinterpret_cast<const uint2*>(op.idx + sl * op.istride) + lane;
-    }
+    ph = reinterpret_cast<const float4*>(op.hi + o0) + lane;
+    pi = reinterpret_cast<const uint2*>(op.idx + sl * op.istride) + lane;
 #pragma unroll
-    for (int d = 0; d < kTileDepth; ++d) fetch(d, first + d * step);
+    for (int d = 0; d < D; ++d) fetch(d, first + d * step);
   }
   // ax,ay,az += sum of a (k - v_a)
   __device__ __forceinline__ void sum(const float4* __restrict__ u, int first, int step, float kx, float ky, float kz,
                                       float& ax, float& ay, float& az) {
-    for (int g0 = first; g0 < ngw; g0 += kTileDepth * step) {
+    for (int g0 = first; g0 < ngw; g0 += D * step) {
 #pragma unroll
-      for (int d = 0; d < kTileDepth; ++d) {
+      for (int d = 0; d < D; ++d) {
         const int g = g0 + d * step;
         if (g < ngw) {
           const float4 ac = a[d];
           const uint2 pc = p[d];
-          fetch(d, g + kTileDepth * step);
+          fetch(d, g + D * step);
           if (g < ng) {
             uint32_t o[4];
             tile_unpack(pc, o);
@@ -136,6 +141,8 @@ struct TileStream {
     }
   }
 };
+
+using TileStream = TileStreamD<kTileDepth>;
 
 // the row's value from its sum, as apply_row
 __device__ __forceinline__ float4 tile_finish(uint8_t kd, float4 vb, float ax, float ay, float az, float sc) {
@@ -166,6 +173,50 @@ __device__ __forceinline__ void tile_combine(float* part, int split, int row, fl
       ay += q[1];
       az += q[2];
     }
+  }
+}
+
+// A row's operator sum in double-float arithmetic over the tile form (residual_row
+// of residual_row.cuh with the gathers from shared memory).  X2: x = hi + lo in two
+// arrays uh, ul; else a float32 vector in uh.
+template <bool X2>
+__device__ __forceinline__ void tile_residual_row(const TileView& op, const float4* uh, const float4* ul, int64_t sl,
+                                                  int lane, int c, int first, int step, float4 kh, float4 kl,
+                                                  DFAcc& a0, DFAcc& a1, DFAcc& a2) {
+  const int64_t o0 = op.off[sl];
+  const float4* __restrict__ ph = reinterpret_cast<const float4*>(op.hi + o0) + lane;
+  const float4* __restrict__ pl = reinterpret_cast<const float4*>(op.lo + o0) + lane;
+  const uint2* __restrict__ pi = reinterpret_cast<const uint2*>(op.idx + sl * op.istride) + lane;
+  const int ng = (c + 3) >> 2;
+  float4 h = make_float4(0.f, 0.f, 0.f, 0.f), l = h;
+  uint2 p = make_uint2(0u, 0u);
+  if (first < ng) {
+    h = __ldcs(ph + first * 32);
+    l = __ldcs(pl + first * 32);
+    p = __ldcs(pi + first * 32);
+  }
+  for (int g = first; g < ng; g += step) {
+    float4 hn = h, ln = l;
+    uint2 pn = p;
+    if (g + step < ng) {
+      hn = __ldcs(ph + (g + step) * 32);
+      ln = __ldcs(pl + (g + step) * 32);
+      pn = __ldcs(pi + (g + step) * 32);
+    }
+    uint32_t o[4];
+    tile_unpack(p, o);
+    const float hv[4] = {h.x, h.y, h.z, h.w}, lv[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float4 xh = tile_at(uh, o[k]);
+      const float4 xl = X2 ? tile_at(ul, o[k]) : make_float4(0.f, 0.f, 0.f, 0.f);
+      a0.add(hv[k], lv[k], kh.x, xh.x, kl.x, xl.x);
+      a1.add(hv[k], lv[k], kh.y, xh.y, kl.y, xl.y);
+      a2.add(hv[k], lv[k], kh.z, xh.z, kl.z, xl.z);
+    }
+    h = hn;
+    l = ln;
+    p = pn;
   }
 }
 

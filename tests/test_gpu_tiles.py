@@ -105,3 +105,55 @@ def test_forms_follow_each_other():
         for x in xs:
             res, _ = oop.true_residual(A, x, s.b)
             assert res <= 1.1e-9
+
+
+@pytest.mark.parametrize("name", ["one_row", "ragged_1", "gaussian", "large_region", "tiles_256", "tiles_128"])
+def test_cooperative_solve_equals_the_launched_loop(name):
+    """The one-kernel solve against the launched loop (which runs while the applies are
+    profiled) and the oracle's matrix: both reach the same true residual, and at 1e-10 the
+    two solutions agree to the residual times the system's conditioning (below 1e3 here)."""
+    torch = torch_cuda()
+    from paper_2206_14780_gb300 import binding
+
+    make, maxnb = CASES[name]
+    s = make()
+    nb, _ = lib_build(s, maxnb)
+    _, _, A = oracle_system(s)
+    b = torch.from_numpy(s.b).cuda()
+    xs = []
+    for profiled in (False, True):
+        nb.profile(profiled)
+        x = torch.from_numpy(s.x0).cuda()
+        rep = nb.solve(params_for(s), binding.solve_opts(rtol=1e-10), b, x)
+        assert rep["status"] == 0 and rep["true_rel_res"] <= 1e-10
+        xs.append(x.cpu().numpy())
+        res, _ = oop.true_residual(A, xs[-1], s.b)
+        assert res <= 1.1e-10
+    assert rel_l2(xs[0], xs[1]) < 1e-7
+
+
+def test_cooperative_solve_limits_and_stalls():
+    """maxit, max_refine, a zero right-hand side and an exact start end the one-kernel solve
+    as they end the loop."""
+    torch = torch_cuda()
+    from paper_2206_14780_gb300 import binding
+
+    s = scenes.couette(5)
+    nb, _ = lib_build(s)
+    b = torch.from_numpy(s.b).cuda()
+    for kw, status in ((dict(maxit=3), 6), (dict(max_refine=1, rtol=1e-10), 6), (dict(), 0)):
+        reps = []
+        for profiled in (False, True):
+            nb.profile(profiled)
+            x = torch.from_numpy(s.x0).cuda()
+            reps.append(nb.solve(params_for(s), binding.solve_opts(**kw), b, x))
+        assert [r["status"] for r in reps] == [status, status]
+        if "maxit" in kw:
+            assert reps[0]["iters"] == reps[1]["iters"] == 3
+        if "max_refine" in kw:
+            assert reps[0]["refinements"] == reps[1]["refinements"] == 1
+    nb.profile(False)
+    zero = torch.zeros_like(b)
+    x = torch.zeros_like(b)
+    rep = nb.solve(params_for(s), binding.solve_opts(), zero, x)
+    assert rep["status"] == 0 and rep["iters"] == 0 and float(x.abs().max()) == 0.0
