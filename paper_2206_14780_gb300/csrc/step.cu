@@ -26,7 +26,9 @@
 #include <cmath>
 #include <cstring>
 
+#include "dfloat.cuh"
 #include "sph_internal.cuh"
+#include "tiles.cuh"
 
 namespace sph {
 
@@ -180,6 +182,192 @@ __global__ void __launch_bounds__(kBlock) k_step_forces(const float4* __restrict
   }
 }
 
+// ---- the two pair sums over the tile form (tiles.cuh) ------------------------------
+// k_step_dummy and k_step_forces walk the 32-bit lists with one thread per row and add
+// in float64 (63 cycles an addition and a conversion): 85 and 149 us on 91k rows, 47
+// and 70 us on 1.4k.  Here the union's data come from shared memory, S = 8 / TS threads
+// share a row, and the sums run in double-float arithmetic (TwoSum; a few 2^-47 of the
+// terms' magnitudes, stored to float32 as before).
+
+struct TileLists {
+  const uint16_t* idx;
+  int64_t istride;
+  const int32_t *uni, *unum, *nfl, *cnt;
+  int32_t ustride, ntiles;
+  int64_t nslices;
+};
+
+TileLists tile_lists(const sph_neighbors* H) {
+  return TileLists{H->t_idx.p,  H->t_istride, H->t_uni.p,    H->t_unum.p,          H->t_nfl.p,
+                   H->cnt.p,    H->t_ustride, (int32_t)H->ntiles, H->nslices};
+}
+
+// running sum: s + e follows the exact sum of the terms
+struct Sum2 {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    float t, r;
+    two_sum(s, x, t, r);
+    s = t;
+    e += r;
+  }
+  __device__ __forceinline__ void add(const Sum2& o) {
+    add(o.s);
+    e += o.e;
+  }
+  __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+};
+
+// dummy walls, as k_step_dummy
+template <int TS>
+__global__ void __launch_bounds__(256) k_tile_dummy(TileLists L, const float4* __restrict__ pos_s, float* rho_s,
+                                                    const uint8_t* __restrict__ type_s, const int32_t* __restrict__ perm,
+                                                    int64_t n, StepGeom g, dfl gx, dfl gy, dfl gz, double rho0, double c0,
+                                                    double zeta, float* P_s, float* __restrict__ rho_c) {
+  constexpr int S = 8 / TS, R = 32 * TS;
+  extern __shared__ __align__(16) float4 dyn[];
+  __shared__ float part[S > 1 ? S - 1 : 1][4][R];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int split = wid / TS, row = (wid % TS) * 32 + lane;
+  for (int64_t tile = blockIdx.x; tile < L.ntiles; tile += gridDim.x) {
+    const int64_t sl = tile * TS + wid % TS, s = sl * kSlice + lane;
+    const bool wall = s < n && type_s[s] != SPH_FLUID;
+    if (__syncthreads_or(wall) == 0) continue;
+    const int nu = L.unum[tile];
+    const int32_t* __restrict__ ids = L.uni + tile * L.ustride;
+    float4 *X = dyn, *Y = dyn + nu;   // x, y, z; P, rho
+    for (int i = tid; i < nu; i += 256) {
+      const int t = ids[i];
+      if (type_s[t] != SPH_FLUID) continue;   // walls are being rewritten; no row reads them
+      X[i] = pos_s[t];
+      Y[i] = make_float4(P_s[t], rho_s[t], 0.f, 0.f);
+    }
+    __syncthreads();
+    const int nf = wall ? L.nfl[s] : 0;
+    const float4 pb = wall ? pos_s[s] : make_float4(0.f, 0.f, 0.f, 0.f);
+    Sum2 W;
+    dfl num{0.f, 0.f};
+    tile_walk(L.idx, L.istride, sl, lane, nf, nf, split, S, [&](uint32_t o) {
+      const float4 pa = tile_at(X, o), q4 = tile_at(Y, o);
+      float d[3] = {pb.x - pa.x, pb.y - pa.y, pb.z - pa.z};   // r_w - r_a
+      min_image(d, g);
+      const float w = kernel_w(sqrtf(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]) * g.inv_h, g);
+      const dfl gr = df_add(df_add(df_mul(gx, dfl{d[0], 0.f}), df_mul(gy, dfl{d[1], 0.f})), df_mul(gz, dfl{d[2], 0.f}));
+      W.add(w);
+      num = df_add(num, df_mul(dfl{w, 0.f}, df_add(dfl{q4.x, 0.f}, df_mul(gr, dfl{q4.y, 0.f}))));
+    });
+    if (S > 1) {
+      if (split > 0) {
+        float(*q)[R] = part[split - 1];
+        q[0][row] = W.s;
+        q[1][row] = W.e;
+        q[2][row] = num.hi;
+        q[3][row] = num.lo;
+      }
+      __syncthreads();
+      if (split == 0)
+        for (int k = 0; k < S - 1; ++k) {
+          W.add(Sum2{part[k][0][row], part[k][1][row]});
+          num = df_add(num, dfl{part[k][2][row], part[k][3][row]});
+        }
+    }
+    if (wall && split == 0) {
+      const double Sw = W.value();
+      const double P = Sw > 0.0 ? df_to_double(num) / Sw : 0.0;
+      const double r = rho0 * pow(P * zeta / (c0 * c0 * rho0) + 1.0, 1.0 / zeta);
+      P_s[s] = (float)P;
+      rho_s[s] = (float)r;
+      rho_c[perm[s]] = (float)r;
+    }
+    __syncthreads();
+  }
+}
+
+// abar and drho/dt, as k_step_forces
+template <int TS>
+__global__ void __launch_bounds__(256) k_tile_forces(TileLists L, const float4* __restrict__ pos_s,
+                                                     const float* __restrict__ rho_s, const uint8_t* __restrict__ type_s,
+                                                     const int32_t* __restrict__ perm, const float4* __restrict__ vel,
+                                                     const float* __restrict__ P_s, int64_t n, StepGeom g, double gx,
+                                                     double gy, double gz, int dummy, float4* __restrict__ acc,
+                                                     float* __restrict__ drho) {
+  constexpr int S = 8 / TS, R = 32 * TS;
+  extern __shared__ __align__(16) float4 dyn[];
+  __shared__ float part[S > 1 ? S - 1 : 1][8][R];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int split = wid / TS, row = (wid % TS) * 32 + lane;
+  for (int64_t tile = blockIdx.x; tile < L.ntiles; tile += gridDim.x) {
+    const int nu = L.unum[tile];
+    const int32_t* __restrict__ ids = L.uni + tile * L.ustride;
+    float4 *X = dyn, *Y = dyn + nu;   // x, y, z, m; u, P / rho^2
+    for (int i = tid; i < nu; i += 256) {
+      const int t = ids[i];
+      const float ra = rho_s[t];
+      float4 u = vel[perm[t]];
+      u.w = P_s[t] / (ra * ra);
+      X[i] = pos_s[t];
+      Y[i] = u;
+    }
+    const int64_t sl = tile * TS + wid % TS, s = sl * kSlice + lane;
+    const bool live = s < n;
+    const bool fluid = live && type_s[s] == SPH_FLUID;
+    const bool on = fluid || (live && !dummy);
+    const int32_t ib = live ? perm[s] : 0;
+    float4 pb = make_float4(0.f, 0.f, 0.f, 0.f), ub = pb;
+    float Pb = 0.f;
+    int nf = 0, c = 0;
+    if (on) {
+      nf = L.nfl[s];
+      c = L.cnt[s];
+      pb = pos_s[s];
+      ub = vel[ib];
+      const float rb = rho_s[s];
+      Pb = P_s[s] / (rb * rb);
+    }
+    __syncthreads();
+    Sum2 ax, ay, az, dr;
+    tile_walk(L.idx, L.istride, sl, lane, nf, c, split, S, [&](uint32_t o) {
+      const float4 pa = tile_at(X, o), ua = tile_at(Y, o);
+      float d[3] = {pa.x - pb.x, pa.y - pb.y, pa.z - pb.z};   // r_a - r_b
+      min_image(d, g);
+      const float q = sqrtf(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]) * g.inv_h;
+      const float mF = pa.w * kernel_absf(q, g);
+      const float cp = mF * (ua.w + Pb);
+      ax.add(-(cp * d[0]));
+      ay.add(-(cp * d[1]));
+      az.add(-(cp * d[2]));
+      dr.add(mF * ((ub.x - ua.x) * d[0] + (ub.y - ua.y) * d[1] + (ub.z - ua.z) * d[2]));
+    });
+    if (S > 1) {
+      if (split > 0) {
+        float(*q)[R] = part[split - 1];
+        q[0][row] = ax.s;
+        q[1][row] = ax.e;
+        q[2][row] = ay.s;
+        q[3][row] = ay.e;
+        q[4][row] = az.s;
+        q[5][row] = az.e;
+        q[6][row] = dr.s;
+        q[7][row] = dr.e;
+      }
+      __syncthreads();
+      if (split == 0)
+        for (int k = 0; k < S - 1; ++k) {
+          ax.add(Sum2{part[k][0][row], part[k][1][row]});
+          ay.add(Sum2{part[k][2][row], part[k][3][row]});
+          az.add(Sum2{part[k][4][row], part[k][5][row]});
+          dr.add(Sum2{part[k][6][row], part[k][7][row]});
+        }
+    }
+    if (live && split == 0) {
+      acc[ib] = fluid ? make_float4((float)(ax.value() + gx), (float)(ay.value() + gy), (float)(az.value() + gz), 0.f)
+                      : make_float4(0.f, 0.f, 0.f, 0.f);
+      drho[ib] = on ? (float)dr.value() : 0.f;
+    }
+    __syncthreads();
+  }
+}
+
 // b = u^n + hdt abar on fluid rows; 2 u_w (dummy) or u_w (dynamic) on walls
 __global__ void k_step_rhs(const float4* __restrict__ u_n, const float4* __restrict__ acc,
                            const uint8_t* __restrict__ type, int64_t n, double hdt, int dummy, double* __restrict__ b) {
@@ -311,21 +499,40 @@ sph_status evaluate(sph_state* S, const sph_step_params* Pp, sph_neighbors** han
   SPH_TRY(T.P_s.alloc(H->n_pad));
   if (Pp->rheology == 1)
     SPH_TRY(mu_papanastasiou(H, S->vel, S->vel, Pp->tau0, Pp->mu0, Pp->m, S->mu, 1, st));
-  SPH_TRY(ensure_nbr(H, st));
+  if (!H->tile_ok) SPH_TRY(ensure_nbr(H, st));
   const StepGeom g = step_geom(H, S);
   const int grid = grid_for(H, H->n);
   SPH_LAUNCH(k_step_eos, grid, kBlock, 0, st)(H->rho_s.p, H->n, Pp->rho0, Pp->c0, Pp->zeta, T.P_s.p);
   const int dummy = Pp->boundary == SPH_BC_DUMMY ? 1 : 0;
+  const float4* vel = reinterpret_cast<const float4*>(S->vel);
+  const size_t smem = tile_smem(H, 32);
+  auto split = [](double x) {
+    const float hi = (float)x;
+    return dfl{hi, (float)(x - (double)hi)};
+  };
   if (dummy) {
-    SPH_LAUNCH(k_step_dummy, grid, kBlock, 0, st)(H->pos_s.p, H->rho_s.p, H->type_s.p, H->cnt.p, H->slice_off.p,
-                                                   H->nbr.p, H->perm.p, H->n, g, Pp->g[0], Pp->g[1], Pp->g[2],
-                                                   Pp->rho0, Pp->c0, Pp->zeta, T.P_s.p, S->rho);
+    if (H->tile_ok) {
+      auto kern = SPH_TILE_PICK(H, k_tile_dummy);
+      SPH_LAUNCH(kern, tile_grid(H, (const void*)kern, smem), 256, smem, st)(
+          tile_lists(H), H->pos_s.p, H->rho_s.p, H->type_s.p, H->perm.p, H->n, g, split(Pp->g[0]), split(Pp->g[1]),
+          split(Pp->g[2]), Pp->rho0, Pp->c0, Pp->zeta, T.P_s.p, S->rho);
+    } else {
+      SPH_LAUNCH(k_step_dummy, grid, kBlock, 0, st)(H->pos_s.p, H->rho_s.p, H->type_s.p, H->cnt.p, H->slice_off.p,
+                                                     H->nbr.p, H->perm.p, H->n, g, Pp->g[0], Pp->g[1], Pp->g[2],
+                                                     Pp->rho0, Pp->c0, Pp->zeta, T.P_s.p, S->rho);
+    }
     H->mu_version++;   // the walls' densities enter A(dt): set it up again
   }
-  SPH_LAUNCH(k_step_forces, grid, kBlock, 0, st)(H->pos_s.p, H->rho_s.p, H->type_s.p, H->cnt.p, H->slice_off.p,
-                                                  H->nbr.p, H->perm.p, reinterpret_cast<const float4*>(S->vel),
-                                                  T.P_s.p, H->n, g, Pp->g[0], Pp->g[1], Pp->g[2], dummy, T.acc.p,
-                                                  T.drho.p);
+  if (H->tile_ok) {
+    auto kern = SPH_TILE_PICK(H, k_tile_forces);
+    SPH_LAUNCH(kern, tile_grid(H, (const void*)kern, smem), 256, smem, st)(
+        tile_lists(H), H->pos_s.p, H->rho_s.p, H->type_s.p, H->perm.p, vel, T.P_s.p, H->n, g, Pp->g[0], Pp->g[1],
+        Pp->g[2], dummy, T.acc.p, T.drho.p);
+  } else {
+    SPH_LAUNCH(k_step_forces, grid, kBlock, 0, st)(H->pos_s.p, H->rho_s.p, H->type_s.p, H->cnt.p, H->slice_off.p,
+                                                    H->nbr.p, H->perm.p, vel, T.P_s.p, H->n, g, Pp->g[0], Pp->g[1],
+                                                    Pp->g[2], dummy, T.acc.p, T.drho.p);
+  }
   SPH_TRY_CUDA(cudaGetLastError());
   return SPH_OK;
 }

@@ -393,11 +393,6 @@ __global__ void __launch_bounds__(256) k_tile_residual(TileView op, const float4
 
 }  // namespace
 
-// one of three instances by the handle's slices per tile
-#define SPH_TILE_PICK(H, name, ...) \
-  ((H)->tile_ts == 8 ? name<8 __VA_ARGS__> : ((H)->tile_ts == 4 ? name<4 __VA_ARGS__> : name<2 __VA_ARGS__>))
-#define SPH_COMMA ,
-
 sph_status tile_fill(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st) {
   SPH_TRY(H->t_hi.alloc(H->t_entries > 0 ? H->t_entries : 1));
   SPH_TRY(H->t_lo.alloc(H->t_entries > 0 ? H->t_entries : 1));

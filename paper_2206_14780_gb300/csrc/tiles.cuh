@@ -144,6 +144,28 @@ struct TileStreamD {
 
 using TileStream = TileStreamD<kTileDepth>;
 
+// f(byte offset of a float4 in the union) for every neighbour of a row, wall neighbours
+// of wall rows included: nf interleaved entries, then c - nf from the next group on.
+// The row's groups first, first + step, ...; the next group's positions are loaded
+// before the current one is worked on.
+template <class F>
+__device__ __forceinline__ void tile_walk(const uint16_t* __restrict__ idx, int64_t istride, int64_t sl, int lane, int nf,
+                                          int c, int first, int step, F f) {
+  const uint2* __restrict__ pi = reinterpret_cast<const uint2*>(idx + sl * istride) + lane;
+  const int gf = (nf + 3) >> 2, ng = gf + ((c - nf + 3) >> 2);
+  uint2 p = first < ng ? pi[first * 32] : make_uint2(0u, 0u);
+  for (int g = first; g < ng; g += step) {
+    const uint2 pn = g + step < ng ? pi[(g + step) * 32] : p;
+    uint32_t o[4];
+    tile_unpack(p, o);
+    const int left = g < gf ? nf - 4 * g : c - nf - 4 * (g - gf);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (k < left) f(o[k]);
+    p = pn;
+  }
+}
+
 // the row's value from its sum, as apply_row
 __device__ __forceinline__ float4 tile_finish(uint8_t kd, float4 vb, float ax, float ay, float az, float sc) {
   if (kd == KIND_FLUID) return make_float4((vb.x + ax) * sc, (vb.y + ay) * sc, (vb.z + az) * sc, 0.f);
@@ -223,6 +245,11 @@ __device__ __forceinline__ void tile_residual_row(const TileView& op, const floa
 TileView tile_view(const sph_neighbors* H);
 // dynamic shared memory of a kernel that holds `bytes_per_row` of every union row
 size_t tile_smem(const sph_neighbors* H, int bytes_per_row);
+// one of a kernel template's three instances, by the handle's slices per tile
+#define SPH_TILE_PICK(H, name, ...) \
+  ((H)->tile_ts == 8 ? name<8 __VA_ARGS__> : ((H)->tile_ts == 4 ? name<4 __VA_ARGS__> : name<2 __VA_ARGS__>))
+#define SPH_COMMA ,
+
 // blocks for a tile kernel: every tile, or as many as are resident at once
 int tile_grid(const sph_neighbors* H, const void* kernel, size_t smem);
 
