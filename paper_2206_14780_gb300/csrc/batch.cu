@@ -13,7 +13,9 @@
 // One refinement pass is four launches: float64 residual per scene (decides on
 // the device which scenes still exceed rtol), pass initialisation, one
 // persistent cooperative kernel that runs all BiCGSTAB iterations of the active
-// scenes with grid barriers between phases, and x += d.  The whole solve is one
+// scenes with grid barriers between phases, and x += d.  Where every scene has the
+// tile form its applies and residuals run on that (16 scenes, 650k rows: 41.2 ->
+// 36.5 ms a solve); the row-loop forms serve the others.  The whole solve is one
 // CUDA graph launch: the pass sits in the body of a conditional WHILE node whose
 // last kernel decides on the device whether another pass follows (some scene
 // still above rtol, passes left, no barrier timed out); where the driver cannot
@@ -21,6 +23,7 @@
 // tile, so the grid keeps working on the scenes that remain.  Every grid
 // barrier spins a bounded number of times and reports SPH_ERR_TIMEOUT instead
 // of hanging.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -31,6 +34,7 @@
 #include "reduce.cuh"
 #include "residual_row.cuh"
 #include "sph_internal.cuh"
+#include "tiles.cuh"
 
 namespace sph {
 
@@ -44,6 +48,8 @@ constexpr float kTileMargin = 0.97f;
 
 struct SceneDesc {
   OpView op;
+  TileView tv;         // the tile form (tiles.cuh), when every scene of the batch has it
+  int32_t ts;          // its slices per tile
   const float* op_lo;
   const double* D64;
   int64_t row_off;     // first row of the scene in the concatenated vectors
@@ -159,6 +165,75 @@ __device__ __forceinline__ void tile_rows(const BatchView& B, int t, int64_t& fi
   end = ((int64_t)B.tile_slice0[t] + B.tile_nsl[t]) * kSlice;
 }
 
+// ---- the tile form inside a batch tile -----------------------------------------------
+// A batch tile of a scene is a run of that scene's tiles (16, 32 and 64 slices are
+// whole numbers of 2, 4 or 8): the block takes them one after the other, each with its
+// union in shared memory and 8 / ts threads per row.
+struct TileLane {
+  int split, splits, row, rows;   // the thread's share of a row and its row in the tile
+  int64_t sl, s;                  // slice and row in the scene
+  bool have;
+};
+__device__ __forceinline__ TileLane tile_lane(const SceneDesc& d, int64_t tile) {
+  TileLane L;
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  L.splits = 8 / d.ts;
+  L.split = wid / d.ts;
+  L.row = (wid % d.ts) * 32 + lane;
+  L.rows = 32 * d.ts;
+  L.sl = tile * d.ts + wid % d.ts;
+  L.s = L.sl * kSlice + lane;
+  L.have = L.sl < d.tv.nslices;
+  return L;
+}
+
+// fin(row, v_b, y) for the rows of batch tile [sl0, sl0 + nsl) of y = D^-1 A v; u: the
+// union, part: [3][64][3] floats
+template <class Fin>
+__device__ __forceinline__ void batch_apply(const SceneDesc& d, const float4* __restrict__ v, int64_t sl0, int nsl,
+                                            float4* u, float* part, Fin fin) {
+  const TileView& op = d.tv;
+  const int lane = threadIdx.x & 31;
+  for (int sub = 0; sub < nsl; sub += d.ts) {
+    const int64_t tile = (sl0 + sub) / d.ts;
+    tile_load_union(op, tile, v, u);
+    const TileLane L = tile_lane(d, tile);
+    int c = 0;
+    uint8_t kd = KIND_IDENTITY;
+    float4 vb = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (L.have) {
+      c = op.cnt[L.s];
+      kd = op.kind[L.s];
+      vb = v[L.s];
+    }
+    const float kap = kd == KIND_FLUID ? 1.f : 0.f;
+    TileStream ts;
+    ts.start(op, L.sl, lane, c, L.split, L.splits);
+    cp_async_wait_all();
+    __syncthreads();
+    float ax = 0.f, ay = 0.f, az = 0.f;
+    ts.sum(u, L.split, L.splits, kap * vb.x, kap * vb.y, kap * vb.z, ax, ay, az);
+    if (L.splits > 1) {
+      if (L.split > 0) {
+        float* q = part + ((L.split - 1) * L.rows + L.row) * 3;
+        q[0] = ax;
+        q[1] = ay;
+        q[2] = az;
+      }
+      __syncthreads();
+      if (L.split == 0)
+        for (int k = 0; k < L.splits - 1; ++k) {
+          const float* q = part + (k * L.rows + L.row) * 3;
+          ax += q[0];
+          ay += q[1];
+          az += q[2];
+        }
+    }
+    if (L.have && L.split == 0) fin(L.s, vb, tile_finish(kd, vb, ax, ay, az, op.invD[L.s]));
+    __syncthreads();
+  }
+}
+
 // ---- residual per scene (double-float pair sums) + which scenes need a pass --
 
 __global__ void __launch_bounds__(kBlock) kb_split(BatchView B, int64_t nrows) {
@@ -171,7 +246,10 @@ __global__ void __launch_bounds__(kBlock) kb_split(BatchView B, int64_t nrows) {
   }
 }
 
+template <bool TILE>
 __global__ void __launch_bounds__(kBlock) kb_residual(BatchView B) {
+  extern __shared__ __align__(16) float4 dyn[];
+  __shared__ double rpart[TILE ? 192 * 3 : 1];
   if (threadIdx.x == 0 && blockIdx.x == 0) {   // counted by kb_init
     B.ctrl->active = 0;
     B.ctrl->passes += 1;
@@ -181,27 +259,79 @@ __global__ void __launch_bounds__(kBlock) kb_residual(BatchView B) {
     const SceneDesc& d = B.sc[sc];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double acc2[3] = {0.0, 0.0, 0.0};
-    for (int w = warp; w < B.tile_nsl[t]; w += kBlock / 32) {
-      const int64_t sl = B.tile_slice0[t] + w;
-      const int64_t s = sl * kSlice + lane;
-      const OpView& op = d.op;
-      const float4* x2 = B.V.x2 + 2 * d.row_off;
-      const uint8_t k = op.kind[s];
-      const float kap = (k == KIND_FLUID) ? 1.f : 0.f;
-      DFAcc a0, a1, a2;
-      residual_row_df(op, d.op_lo, x2, sl, lane, kap, a0, a1, a2);
+    auto finish = [&](int64_t s, uint8_t k, double v0, double v1, double v2) {
       const double sg = (k == KIND_FLUID) ? 1.0 : (k == KIND_SHEPARD ? -1.0 : 0.0);
       const int64_t g = d.row_off + s;
       double r[3] = {0.0, 0.0, 0.0};
       if (s < d.n) {
-        r[0] = B.V.b64[3 * g] - (B.V.x64[3 * g] + sg * a0.value());
-        r[1] = B.V.b64[3 * g + 1] - (B.V.x64[3 * g + 1] + sg * a1.value());
-        r[2] = B.V.b64[3 * g + 2] - (B.V.x64[3 * g + 2] + sg * a2.value());
+        r[0] = B.V.b64[3 * g] - (B.V.x64[3 * g] + sg * v0);
+        r[1] = B.V.b64[3 * g + 1] - (B.V.x64[3 * g + 1] + sg * v1);
+        r[2] = B.V.b64[3 * g + 2] - (B.V.x64[3 * g + 2] + sg * v2);
       }
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         B.V.r64[3 * g + q] = r[q];
         acc2[q] += r[q] * r[q];
+      }
+    };
+    const float4* x2 = B.V.x2 + 2 * d.row_off;
+    if (TILE) {
+      for (int sub = 0; sub < B.tile_nsl[t]; sub += d.ts) {
+        const int64_t tile = (B.tile_slice0[t] + sub) / d.ts;
+        const int nu = d.tv.unum[tile];
+        const int32_t* __restrict__ ids = d.tv.uni + tile * d.tv.ustride;
+        float4 *uh = dyn, *ul = dyn + nu;
+        for (int i = threadIdx.x; i < nu; i += kBlock) {
+          const int64_t q = ids[i];
+          cp_async16(uh + i, x2 + 2 * q);
+          cp_async16(ul + i, x2 + 2 * q + 1);
+        }
+        const TileLane L = tile_lane(d, tile);
+        int c = 0;
+        uint8_t k = KIND_IDENTITY;
+        float4 bh = make_float4(0.f, 0.f, 0.f, 0.f), bl = bh;
+        if (L.have) {
+          c = d.tv.cnt[L.s];
+          k = d.tv.kind[L.s];
+          bh = x2[2 * L.s];
+          bl = x2[2 * L.s + 1];
+        }
+        const float kap = k == KIND_FLUID ? 1.f : 0.f;
+        cp_async_wait_all();
+        __syncthreads();
+        DFAcc a0, a1, a2;
+        if (c > 0)
+          tile_residual_row<true>(d.tv, uh, ul, L.sl, lane, c, L.split, L.splits,
+                                  make_float4(kap * bh.x, kap * bh.y, kap * bh.z, 0.f),
+                                  make_float4(kap * bl.x, kap * bl.y, kap * bl.z, 0.f), a0, a1, a2);
+        double v0 = a0.value(), v1 = a1.value(), v2 = a2.value();
+        if (L.splits > 1) {
+          if (L.split > 0) {
+            double* q = rpart + ((L.split - 1) * L.rows + L.row) * 3;
+            q[0] = v0;
+            q[1] = v1;
+            q[2] = v2;
+          }
+          __syncthreads();
+          if (L.split == 0)
+            for (int w = 0; w < L.splits - 1; ++w) {
+              const double* q = rpart + (w * L.rows + L.row) * 3;
+              v0 += q[0];
+              v1 += q[1];
+              v2 += q[2];
+            }
+        }
+        if (L.have && L.split == 0) finish(L.s, k, v0, v1, v2);
+        __syncthreads();
+      }
+    } else {
+      for (int w = warp; w < B.tile_nsl[t]; w += kBlock / 32) {
+        const int64_t sl = B.tile_slice0[t] + w;
+        const int64_t s = sl * kSlice + lane;
+        const uint8_t k = d.op.kind[s];
+        DFAcc a0, a1, a2;
+        residual_row_df(d.op, d.op_lo, x2, sl, lane, (k == KIND_FLUID) ? 1.f : 0.f, a0, a1, a2);
+        finish(s, k, a0.value(), a1.value(), a2.value());
       }
     }
     block_partials_f64<3>(acc2, B.partials + (size_t)t * kMaxDots);
@@ -271,8 +401,10 @@ __global__ void __launch_bounds__(kBlock) kb_init(BatchView B) {
 
 // One BiCGSTAB pass for every active scene: loops over iterations until no
 // scene progresses, with a grid barrier between the phases of an iteration.
-template <int U, bool PF, int NB>
-__global__ void __launch_bounds__(NB) kb_pass(BatchView B, int iter_cap) {
+template <int U, bool PF, int NB, bool TILE>
+__global__ void __launch_bounds__(NB, TILE ? 4 : 1) kb_pass(BatchView B, int iter_cap) {
+  extern __shared__ __align__(16) float4 dyn[];
+  __shared__ float part[TILE ? 192 * 3 : 1];
   for (int it = 0; it < iter_cap; ++it) {
     if (*(volatile int32_t*)&B.ctrl->active == 0) break;
     // phase 1: p = r + beta p - alpha' Ap
@@ -281,8 +413,8 @@ __global__ void __launch_bounds__(NB) kb_pass(BatchView B, int iter_cap) {
       const SolverScalars* S = B.S + sc;
       if (S->done) continue;
       const SceneDesc& d = B.sc[sc];
-      const float b0 = (float)S->beta[0], b1 = (float)S->beta[1], b2 = (float)S->beta[2];
-      const float a0 = (float)S->alpha_p[0], a1 = (float)S->alpha_p[1], a2 = (float)S->alpha_p[2];
+      const float b0 = S->beta_f[0], b1 = S->beta_f[1], b2 = S->beta_f[2];
+      const float a0 = S->alphap_f[0], a1 = S->alphap_f[1], a2 = S->alphap_f[2];
       const bool useP = b0 != 0.f || b1 != 0.f || b2 != 0.f, useA = a0 != 0.f || a1 != 0.f || a2 != 0.f;
       int64_t s0, s1;
       tile_rows(B, t, s0, s1);
@@ -313,17 +445,24 @@ __global__ void __launch_bounds__(NB) kb_pass(BatchView B, int iter_cap) {
       if (S->done) continue;
       const SceneDesc& d = B.sc[sc];
       float acc[3] = {0.f, 0.f, 0.f};
-      const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-      for (int w = warp; w < B.tile_nsl[t]; w += NB / 32) {
-        const int64_t sl = B.tile_slice0[t] + w;
-        float4 vb;
-        const float4 o = apply_row<U, PF, true>(d.op, B.V.p + d.row_off, sl, lane, vb);
-        const int64_t g = d.row_off + sl * kSlice + lane;
+      auto fin = [&](int64_t s, float4, float4 o) {
+        const int64_t g = d.row_off + s;
         B.V.Ap[g] = o;
         const float4 h = B.V.rh[g];
         acc[0] = fmaf(h.x, o.x, acc[0]);
         acc[1] = fmaf(h.y, o.y, acc[1]);
         acc[2] = fmaf(h.z, o.z, acc[2]);
+      };
+      if (TILE) {
+        batch_apply(d, B.V.p + d.row_off, B.tile_slice0[t], B.tile_nsl[t], dyn, part, fin);
+      } else {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        for (int w = warp; w < B.tile_nsl[t]; w += NB / 32) {
+          const int64_t sl = B.tile_slice0[t] + w;
+          float4 vb;
+          const float4 o = apply_row<U, PF, true>(d.op, B.V.p + d.row_off, sl, lane, vb);
+          fin(sl * kSlice + lane, vb, o);
+        }
       }
       block_partials<3, NB>(acc, B.partials + (size_t)t * kMaxDots);
       if (arrive_scene(B.scene_cnt + sc, d.tile_end - d.tile_begin)) {
@@ -339,7 +478,7 @@ __global__ void __launch_bounds__(NB) kb_pass(BatchView B, int iter_cap) {
       const SolverScalars* S = B.S + sc;
       if (S->done) continue;
       const SceneDesc& d = B.sc[sc];
-      const float a0 = (float)S->alpha[0], a1 = (float)S->alpha[1], a2 = (float)S->alpha[2];
+      const float a0 = S->alpha_f[0], a1 = S->alpha_f[1], a2 = S->alpha_f[2];
       int64_t s0, s1;
       tile_rows(B, t, s0, s1);
       for (int64_t s = s0; s < s1; s += NB) {
@@ -356,19 +495,25 @@ __global__ void __launch_bounds__(NB) kb_pass(BatchView B, int iter_cap) {
       if (S->done) continue;
       const SceneDesc& d = B.sc[sc];
       float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-      for (int w = warp; w < B.tile_nsl[t]; w += NB / 32) {
-        const int64_t sl = B.tile_slice0[t] + w;
-        float4 vb;
-        const float4 o = apply_row<U, PF, true>(d.op, B.V.rs + d.row_off, sl, lane, vb);
-        const int64_t g = d.row_off + sl * kSlice + lane;
-        B.V.As[g] = o;
+      auto fin = [&](int64_t s, float4 vb, float4 o) {
+        B.V.As[d.row_off + s] = o;
         acc[0] = fmaf(vb.x, o.x, acc[0]);
         acc[1] = fmaf(vb.y, o.y, acc[1]);
         acc[2] = fmaf(vb.z, o.z, acc[2]);
         acc[3] = fmaf(o.x, o.x, acc[3]);
         acc[4] = fmaf(o.y, o.y, acc[4]);
         acc[5] = fmaf(o.z, o.z, acc[5]);
+      };
+      if (TILE) {
+        batch_apply(d, B.V.rs + d.row_off, B.tile_slice0[t], B.tile_nsl[t], dyn, part, fin);
+      } else {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        for (int w = warp; w < B.tile_nsl[t]; w += NB / 32) {
+          const int64_t sl = B.tile_slice0[t] + w;
+          float4 vb;
+          const float4 o = apply_row<U, PF, true>(d.op, B.V.rs + d.row_off, sl, lane, vb);
+          fin(sl * kSlice + lane, vb, o);
+        }
       }
       block_partials<6, NB>(acc, B.partials + (size_t)t * kMaxDots);
       if (arrive_scene(B.scene_cnt + sc, d.tile_end - d.tile_begin)) {
@@ -385,8 +530,8 @@ __global__ void __launch_bounds__(NB) kb_pass(BatchView B, int iter_cap) {
       if (S->done) continue;
       const SceneDesc& d = B.sc[sc];
       float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      const float w0 = (float)S->omega[0], w1 = (float)S->omega[1], w2 = (float)S->omega[2];
-      const float l0 = (float)S->alpha[0], l1 = (float)S->alpha[1], l2 = (float)S->alpha[2];
+      const float w0 = S->omega_f[0], w1 = S->omega_f[1], w2 = S->omega_f[2];
+      const float l0 = S->alpha_f[0], l1 = S->alpha_f[1], l2 = S->alpha_f[2];
       int64_t s0, s1;
       tile_rows(B, t, s0, s1);
       for (int64_t s = s0; s < s1; s += NB) {
@@ -456,42 +601,37 @@ __global__ void kb_scatter(const double* __restrict__ src, const int32_t* __rest
   }
 }
 
-__global__ void kb_norm2(const double* __restrict__ b, int64_t n_pad, double* out) {
-  // one block per scene (b points at the scene's rows); float64 squares per component
+// squares per component of every scene's b: kNormBlocks blocks per scene, their sums in
+// [scene][block][3] (added up by the host in that order).  One block per scene was
+// bound by one SM's float64 rate: 44 us a scene, one after the other.
+constexpr int kNormBlocks = 32;
+__global__ void __launch_bounds__(kBlock) kb_norm2(const SceneDesc* __restrict__ sc, const double* __restrict__ b64,
+                                                   double* __restrict__ out) {
+  const int scene = blockIdx.x / kNormBlocks, part = blockIdx.x % kNormBlocks;
+  const double* __restrict__ b = b64 + 3 * sc[scene].row_off;
   double acc[3] = {0.0, 0.0, 0.0};
-  for (int64_t i = threadIdx.x; i < n_pad; i += blockDim.x) {
+  for (int64_t i = part * kBlock + threadIdx.x; i < sc[scene].n; i += kNormBlocks * kBlock) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) acc[k] = fma(b[3 * i + k], b[3 * i + k], acc[k]);
   }
-  __shared__ double sm[kBlock / 32][3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    double x = acc[k];
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5][k] = x;
-  }
-  __syncthreads();
-  if (threadIdx.x < 3) {
-    double s = 0.0;
-    for (int w = 0; w < kBlock / 32; ++w) s += sm[w][threadIdx.x];
-    out[threadIdx.x] = s;
-  }
+  block_partials_f64<3>(acc, out + 3 * (size_t)blockIdx.x);
 }
 
 // variants 0..7: row-loop form (v & 3: (U, PF) = (8,0), (4,0), (8,1), (4,1)) and
 // block size (v >> 2: 256 or 128 threads, 8 or 4 warps per 32-slice tile)
 constexpr int kPassVariants = 8;
 using PassFn = void (*)(BatchView, int);
-PassFn pass_kernel(int variant) {
+PassFn pass_kernel(int variant, bool tile) {
+  if (tile) return kb_pass<8, false, 256, true>;
   switch (variant) {
-    case 1: return kb_pass<4, false, 256>;
-    case 2: return kb_pass<8, true, 256>;
-    case 3: return kb_pass<4, true, 256>;
-    case 4: return kb_pass<8, false, 128>;
-    case 5: return kb_pass<4, false, 128>;
-    case 6: return kb_pass<8, true, 128>;
-    case 7: return kb_pass<4, true, 128>;
-    default: return kb_pass<8, false, 256>;
+    case 1: return kb_pass<4, false, 256, false>;
+    case 2: return kb_pass<8, true, 256, false>;
+    case 3: return kb_pass<4, true, 256, false>;
+    case 4: return kb_pass<8, false, 128, false>;
+    case 5: return kb_pass<4, false, 128, false>;
+    case 6: return kb_pass<8, true, 128, false>;
+    case 7: return kb_pass<4, true, 128, false>;
+    default: return kb_pass<8, false, 256, false>;
   }
 }
 int pass_block(int variant) { return (variant >> 2) == 1 ? 128 : 256; }
@@ -508,6 +648,9 @@ struct sph_batch {
   std::vector<sph_visc_params> params;
   std::vector<int64_t> row_off;
   std::vector<uint64_t> rs_version;   // each handle's row-scale version at creation
+  bool tile_form = false;             // every scene's operator is in the tile form
+  size_t smem = 0, smem_res = 0;      // dynamic shared memory of the pass and the residual kernels
+  DBuf<double> norms;                 // [nscenes][kNormBlocks][3]
   int64_t nrows = 0;
   int32_t ntiles = 0;
   int device = 0, num_sms = 0;
@@ -568,7 +711,7 @@ BatchView batch_view(sph_batch* Bt, double rtol, double eps) {
 }
 
 sph_status launch_pass(sph_batch* Bt, const BatchView& B, int cap, cudaStream_t st) {
-  const PassFn kern = pass_kernel(Bt->variant < 0 ? 0 : Bt->variant);
+  const PassFn kern = pass_kernel(Bt->variant < 0 ? 0 : Bt->variant, Bt->tile_form);
   BatchView bv = B;
   int c = cap;
   void* args[] = {&bv, &c};
@@ -576,7 +719,7 @@ sph_status launch_pass(sph_batch* Bt, const BatchView& B, int cap, cudaStream_t 
   const int var = Bt->variant < 0 ? 0 : Bt->variant;
   cfg.gridDim = dim3(Bt->grids[var]);
   cfg.blockDim = dim3(pass_block(var));
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = Bt->smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -592,7 +735,8 @@ sph_status launch_pass(sph_batch* Bt, const BatchView& B, int cap, cudaStream_t 
 sph_status enqueue_pass(sph_batch* Bt, const BatchView& B, int cap, cudaStream_t st) {
   const int g = Bt->grid;
   SPH_LAUNCH(kb_split, g, kBlock, 0, st)(B, Bt->nrows);
-  SPH_LAUNCH(kb_residual, g, kBlock, 0, st)(B);
+  auto residual = Bt->tile_form ? kb_residual<true> : kb_residual<false>;
+  SPH_LAUNCH(residual, g, kBlock, Bt->smem_res, st)(B);
   SPH_LAUNCH(kb_init, g, kBlock, 0, st)(B);
   SPH_TRY(launch_pass(Bt, B, cap, st));
   SPH_LAUNCH(kb_add, g, kBlock, 0, st)(B, Bt->nrows);
@@ -661,13 +805,15 @@ sph_status sph_batch_create(sph_neighbors* const* handles, const sph_visc_params
   Bt->nscenes = nscenes;
   Bt->hdesc.assign(nscenes, SceneDesc{});
   int64_t rows = 0, max_tiles = 0;
+  Bt->tile_form = true;
+  for (int s = 0; s < nscenes; ++s) Bt->tile_form = Bt->tile_form && handles[s] && handles[s]->tile_ok;
   for (int s = 0; s < nscenes; ++s) {
     sph_neighbors* H = handles[s];
     if (!H) {
       set_error("sph_batch_create: handle %d is null", s);
       return fail(SPH_ERR_INVALID);
     }
-    sph_status e = ensure_operator(H, &params[s], st, OP_IH);
+    sph_status e = ensure_operator(H, &params[s], st, Bt->tile_form ? OP_FAST : OP_IH);
     if (e == SPH_OK) e = row_scale_refresh(H, st);
     if (e != SPH_OK) return fail(e);
     Bt->handles.push_back(H);
@@ -678,8 +824,14 @@ sph_status sph_batch_create(sph_neighbors* const* handles, const sph_visc_params
     d.op = op_view(H);
     d.op_lo = H->op_lo.p;
     d.D64 = H->D64.p;
+    if (Bt->tile_form) {
+      d.tv = tile_view(H);
+      d.ts = H->tile_ts;
+      Bt->smem = std::max(Bt->smem, tile_smem(H, 16));
+      Bt->smem_res = std::max(Bt->smem_res, tile_smem(H, 32));
+    }
     if (H->row_scaled) {  // the preconditioner's diagonal D / s
-      d.op.invD = H->invD_sc.p;
+      d.op.invD = d.tv.invD = H->invD_sc.p;
       d.D64 = H->D64_sc.p;
     }
     d.row_off = rows;
@@ -707,6 +859,7 @@ sph_status sph_batch_create(sph_neighbors* const* handles, const sph_visc_params
   BTRY(Bt->S.alloc(nscenes));
   BTRY(Bt->partials.alloc((size_t)max_tiles * kMaxDots));
   BTRY(Bt->rr64.alloc(3 * nscenes));
+  BTRY(Bt->norms.alloc((size_t)3 * kNormBlocks * nscenes));
   BTRY(Bt->scene_cnt.alloc(nscenes));
   BTRY(Bt->iters.alloc(nscenes));
   BTRY(Bt->passes.alloc(nscenes));
@@ -724,7 +877,13 @@ sph_status sph_batch_create(sph_neighbors* const* handles, const sph_visc_params
   // grid of each cooperative variant: every block resident at once
   for (int v = 0; v < kPassVariants; ++v) {
     int o = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, (const void*)pass_kernel(v), pass_block(v), 0);
+    const void* k = (const void*)pass_kernel(v, Bt->tile_form);
+    if (Bt->tile_form) {
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (kTileUnion + 1) * 16);
+      cudaFuncSetAttribute((const void*)kb_residual<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (kTileUnion + 1) * 32);
+    }
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, pass_block(Bt->tile_form ? 0 : v), Bt->smem);
     Bt->occ[v] = o;
   }
   BTRY(build_tiles(Bt, kTileDefault, st));
@@ -746,6 +905,7 @@ sph_status sph_batch_destroy(sph_batch* Bt) {
   Bt->S.release();
   Bt->partials.release();
   Bt->rr64.release();
+  Bt->norms.release();
   Bt->scene_cnt.release();
   Bt->iters.release();
   Bt->passes.release();
@@ -785,7 +945,7 @@ sph_status sph_batch_solve(sph_batch* Bt, const sph_solve_opts* O, const double*
     }
     sph_neighbors* H = Bt->handles[s];
     // the operator may have been rebuilt since the batch was made
-    if (!H->op_valid || H->op_mu_version != H->mu_version || H->rs_version != Bt->rs_version[s] ||
+    if (!H->op_valid || !(Bt->tile_form ? H->op_tile_valid : H->op_ih_valid) || H->op_mu_version != H->mu_version || H->rs_version != Bt->rs_version[s] ||
         (H->row_scaled && H->rs_op_version != H->op_version)) {
       set_error("sph_batch_solve: scene %d's handle changed after sph_batch_create", s);
       return SPH_ERR_INVALID;
@@ -794,13 +954,16 @@ sph_status sph_batch_solve(sph_batch* Bt, const sph_solve_opts* O, const double*
     SPH_LAUNCH(kb_gather, grid_for(H, H->n_pad), kBlock, 0, st)(b[s], H->perm.p, H->n, H->n_pad,
                                                                   Bt->dvec.p + 3 * N + 3 * o);
     SPH_LAUNCH(kb_gather, grid_for(H, H->n_pad), kBlock, 0, st)(x[s], H->perm.p, H->n, H->n_pad, Bt->dvec.p + 3 * o);
-    SPH_LAUNCH(kb_norm2, 1, kBlock, 0, st)(Bt->dvec.p + 3 * N + 3 * o, H->n_pad, Bt->rr64.p + 3 * s);
   }
+  SPH_LAUNCH(kb_norm2, S * kNormBlocks, kBlock, 0, st)(Bt->desc.p, Bt->dvec.p + 3 * N, Bt->norms.p);
   SPH_TRY_CUDA(cudaGetLastError());
   // per-scene ||b||^2 into the descriptors, counters and reports cleared
-  std::vector<double> rr(3 * S);
-  SPH_TRY_CUDA(cudaMemcpyAsync(rr.data(), Bt->rr64.p, 3 * S * sizeof(double), cudaMemcpyDeviceToHost, st));
+  std::vector<double> rr(3 * S, 0.0), parts((size_t)3 * kNormBlocks * S);
+  SPH_TRY_CUDA(cudaMemcpyAsync(parts.data(), Bt->norms.p, parts.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
   SPH_TRY_CUDA(cudaStreamSynchronize(st));
+  for (int s = 0; s < S; ++s)
+    for (int k = 0; k < kNormBlocks; ++k)
+      for (int c = 0; c < 3; ++c) rr[3 * s + c] += parts[((size_t)s * kNormBlocks + k) * 3 + c];
   std::vector<double> bb(S), bbc(3 * S);
   for (int s = 0; s < S; ++s) {
     for (int c = 0; c < 3; ++c) bbc[3 * s + c] = rr[3 * s + c];
@@ -848,7 +1011,8 @@ sph_status sph_batch_solve(sph_batch* Bt, const sph_solve_opts* O, const double*
     sph_status ts = SPH_OK;
     float best = 1e30f;
     int bestv = 0;
-    for (int v = 0; v < kPassVariants && ts == SPH_OK; ++v) {
+    // (the tile form has one row loop and block size: variant 0, timed once)
+    for (int v = 0; v < (Bt->tile_form ? 1 : kPassVariants) && ts == SPH_OK; ++v) {
       Bt->variant = v;
       float ms = 0.f;
       ts = time_pass(ms);

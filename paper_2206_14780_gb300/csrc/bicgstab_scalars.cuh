@@ -21,6 +21,7 @@ constexpr double kFltMin = 1.17549435082228750797e-38;  // 2^-126: the tau^2 flo
 __device__ inline void scal_delta_c(SolverScalars* S, const double* dots, int c) {
   if (S->state[c] != SPH_PROGRESSING) {
     S->alpha[c] = 0.0;
+    S->alpha_f[c] = 0.f;
     S->stall_now[c] = 0;
     return;
   }
@@ -38,18 +39,21 @@ __device__ inline void scal_delta_c(SolverScalars* S, const double* dots, int c)
     }
   }
   S->alpha[c] = a;
+  S->alpha_f[c] = (float)a;
   S->stall_now[c] = stall;
 }
 
 __device__ inline void scal_omega_c(SolverScalars* S, const double* dots, int c) {
   if (S->state[c] != SPH_PROGRESSING) {
     S->omega[c] = 0.0;
+    S->omega_f[c] = 0.f;
     return;
   }
   const double sA = dots[c], AA = dots[3 + c];
   double om = (AA > 0.0 && isfinite(AA)) ? sA / AA : 0.0;
   if (!isfinite(om)) om = 0.0;
   S->omega[c] = om;
+  S->omega_f[c] = (float)om;
 }
 
 // gamma' and r.r of component c known: alpha', beta and its state (returned)
@@ -57,6 +61,7 @@ __device__ inline int scal_update_c(SolverScalars* S, const double* gam_new, con
   if (S->state[c] != SPH_PROGRESSING) {
     S->alpha_p[c] = 0.0;
     S->beta[c] = 0.0;
+    S->alphap_f[c] = S->beta_f[c] = 0.f;
     return S->state[c];
   }
   const double om = S->omega[c];
@@ -70,6 +75,8 @@ __device__ inline int scal_update_c(SolverScalars* S, const double* gam_new, con
   if (!isfinite(gam_new[c]) || !isfinite(rr[c])) S->nonfinite = 1;
   S->alpha_p[c] = ap;
   S->beta[c] = be;
+  S->alphap_f[c] = (float)ap;
+  S->beta_f[c] = (float)be;
   S->gamma[c] = gam_new[c];
   S->rr[c] = rr[c];
   int st;
@@ -125,6 +132,7 @@ __device__ inline void scal_init(SolverScalars* S, const double* g, double eps2,
     S->rr[c] = g[c];
     S->tau2[c] = fmax(eps2 * g[c], kFltMin);
     S->alpha[c] = S->alpha_p[c] = S->beta[c] = S->omega[c] = S->delta[c] = 0.0;
+    S->alpha_f[c] = S->alphap_f[c] = S->beta_f[c] = S->omega_f[c] = 0.f;
     S->stall_now[c] = 0;
     S->stalled_any[c] = 0;
     const int st = (g[c] == 0.0 || g[c] < S->tau2[c]) ? SPH_CONVERGED : SPH_PROGRESSING;
@@ -149,6 +157,7 @@ __device__ inline void scal_init(SolverScalars* S, const double* g, double eps2,
 __device__ inline void scal_cg_alpha_c(SolverScalars* S, const double* dots, int c) {
   if (S->state[c] != SPH_PROGRESSING) {
     S->alpha[c] = 0.0;
+    S->alpha_f[c] = 0.f;
     S->stall_now[c] = 0;
     return;
   }
@@ -157,18 +166,21 @@ __device__ inline void scal_cg_alpha_c(SolverScalars* S, const double* dots, int
   double a = (d != 0.0 && isfinite(d)) ? S->gamma[c] / d : 0.0;
   if (!isfinite(a)) a = 0.0;
   S->alpha[c] = a;
+  S->alpha_f[c] = (float)a;
   S->stall_now[c] = a == 0.0 ? 1 : 0;
 }
 
 __device__ inline int scal_cg_update_c(SolverScalars* S, const double* gam_new, const double* rr, int c) {
   if (S->state[c] != SPH_PROGRESSING) {
     S->beta[c] = 0.0;
+    S->beta_f[c] = 0.f;
     return S->state[c];
   }
   double be = S->stall_now[c] ? 0.0 : gam_new[c] / S->gamma[c];
   if (!isfinite(be)) be = 0.0;
   if (!isfinite(gam_new[c]) || !isfinite(rr[c])) S->nonfinite = 1;
   S->beta[c] = be;
+  S->beta_f[c] = (float)be;
   S->gamma[c] = gam_new[c];
   S->rr[c] = rr[c];
   int st;
@@ -203,6 +215,7 @@ __device__ inline void scal_cg_init(SolverScalars* S, const double* gz, const do
     S->rr[c] = rr[c];
     S->tau2[c] = fmax(eps2 * rr[c], kFltMin);
     S->alpha[c] = S->alpha_p[c] = S->beta[c] = S->omega[c] = S->delta[c] = 0.0;
+    S->alpha_f[c] = S->alphap_f[c] = S->beta_f[c] = S->omega_f[c] = 0.f;
     S->stall_now[c] = 0;
     S->stalled_any[c] = 0;
     const int st = (rr[c] == 0.0 || rr[c] < S->tau2[c]) ? SPH_CONVERGED : SPH_PROGRESSING;

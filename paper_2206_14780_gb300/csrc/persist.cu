@@ -71,7 +71,6 @@ struct PersistArgs {
 struct Shared {
   SolverScalars S;
   double res[6], own[6], rr[3];
-  float f[12];                       // alpha, omega, alpha', beta in float32
   float wsum[kPW][6];
   double wsumd[kPW][6];
   int64_t soff[kPSliceMax];
@@ -337,12 +336,9 @@ __global__ void __launch_bounds__(kPT, 1) k_persist(PersistArgs A) {
               a3[2] = fmaf(h.z, o.z, a3[2]);
             });
       if (!grid_sum<3>(A, epoch, &sh, a3, SP == 1 || rows_here)) return;
-      if (wid == 0) {
-        scal_after_delta_w(S, sh.res);
-        if (lane < 3) sh.f[lane] = (float)S->alpha[lane];
-      }
+      if (wid == 0) scal_after_delta_w(S, sh.res);
       __syncthreads();
-      const float al0 = sh.f[0], al1 = sh.f[1], al2 = sh.f[2];
+      const float al0 = S->alpha_f[0], al1 = S->alpha_f[1], al2 = S->alpha_f[2];
       // r* = r - alpha A p, A r*, omega
 #pragma unroll 2
       for (int i = tid; i < U; i += kPT) {
@@ -368,12 +364,9 @@ __global__ void __launch_bounds__(kPT, 1) k_persist(PersistArgs A) {
         a6[5] = fmaf(o.z, o.z, a6[5]);
       });
       if (!grid_sum<6>(A, epoch, &sh, a6, SP == 1 || rows_here)) return;
-      if (wid == 0) {
-        scal_after_omega_w(S, sh.res);
-        if (lane < 3) sh.f[3 + lane] = (float)S->omega[lane];
-      }
+      if (wid == 0) scal_after_omega_w(S, sh.res);
       __syncthreads();
-      const float w0 = sh.f[3], w1 = sh.f[4], w2 = sh.f[5];
+      const float w0 = S->omega_f[0], w1 = S->omega_f[1], w2 = S->omega_f[2];
       // r = r* - omega A r*, d, gamma' and r.r
 #pragma unroll
       for (int k = 0; k < 6; ++k) a6[k] = 0.f;
@@ -404,17 +397,12 @@ __global__ void __launch_bounds__(kPT, 1) k_persist(PersistArgs A) {
         R[i] = v;
       }
       if (!grid_sum<6>(A, epoch, &sh, a6, rows_here)) return;
-      if (wid == 0) {
-        scal_after_update_w(S, sh.res, sh.res + 3);
-        if (lane < 3) {
-          sh.f[6 + lane] = (float)S->alpha_p[lane];
-          sh.f[9 + lane] = (float)S->beta[lane];
-        }
-      }
+      if (wid == 0) scal_after_update_w(S, sh.res, sh.res + 3);
       __syncthreads();
       if (S->done) break;
       // p = r + beta p - alpha' A p  (a zero coefficient skips its vector)
-      const float c0 = sh.f[6], c1 = sh.f[7], c2 = sh.f[8], b0 = sh.f[9], b1 = sh.f[10], b2 = sh.f[11];
+      const float c0 = S->alphap_f[0], c1 = S->alphap_f[1], c2 = S->alphap_f[2];
+      const float b0 = S->beta_f[0], b1 = S->beta_f[1], b2 = S->beta_f[2];
       const bool useP = (b0 != 0.f) || (b1 != 0.f) || (b2 != 0.f);
       const bool useA = (c0 != 0.f) || (c1 != 0.f) || (c2 != 0.f);
       auto next_p = [&](float4 v, float4 q, float4 a) {

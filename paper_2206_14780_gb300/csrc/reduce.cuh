@@ -17,14 +17,14 @@ namespace sph {
 // out[k] = sum over the W warps of sm[w][k] (k < K), as a shuffle tree inside
 // groups of W consecutive lanes: log2(W) dependent float64 additions instead of
 // W - 1.  Every thread of the block calls it (the first warps do the work).
-template <int K, int W>
-__device__ __forceinline__ void cross_warp_sum(const double (*sm)[K > 0 ? K : 1], double* __restrict__ out) {
+template <int K, int W, class T>
+__device__ __forceinline__ void cross_warp_sum(const T (*sm)[K > 0 ? K : 1], double* __restrict__ out) {
   constexpr int N = K * W;
   constexpr int NT = (N + 31) / 32 * 32;
   static_assert(32 % W == 0, "W must divide the warp");
   const int t = threadIdx.x;
   if (t < NT) {
-    double x = t < N ? sm[t % W][t / W] : 0.0;
+    double x = t < N ? (double)sm[t % W][t / W] : 0.0;
 #pragma unroll
     for (int o = W / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     if (t < N && t % W == 0) out[t / W] = x;
@@ -66,16 +66,18 @@ __device__ __forceinline__ double warp_sum_multi(const double (&in)[K], int& ind
   return v[0];
 }
 
+// The warps' float32 sums go to float64 in cross_warp_sum's one conversion per value
+// (a conversion by every warp costs 63 cycles each).
 template <int K, int NB = kBlock>
 __device__ __forceinline__ void block_partials(const float (&v)[K], double* __restrict__ out) {
-  __shared__ double sm[NB / 32][K > 0 ? K : 1];
+  __shared__ float sm[NB / 32][K > 0 ? K : 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     float x = v[k];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0) sm[warp][k] = (double)x;
+    if (lane == 0) sm[warp][k] = x;
   }
   __syncthreads();
   cross_warp_sum<K, NB / 32>(sm, out);
@@ -115,45 +117,32 @@ __device__ __forceinline__ bool arrive_last(unsigned int* counter) {
 }
 
 // Sum of all block partials (called by every thread of the last block); the
-// result is left in res[0..K) in shared memory; the counter is re-armed.
+// result is left in res[0..K) in shared memory; the counter is re-armed.  Warp k
+// sums value k (k, k + 8, ...): lane l takes blocks l, l + 32, ... (kAhead of them
+// loaded before any is added), then a shuffle tree.  An addition takes a warp 63
+// cycles, so no lane adds for blocks that are not there: at 6 blocks the tail is 5
+// additions per value, where a fixed number of rounds per thread took 27.
 template <int K>
 __device__ __forceinline__ void final_sum(const double* partials, unsigned int* counter, double* res) {
-  double acc[K];
+  constexpr int kAhead = 8;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = (int)gridDim.x;
+  for (int k = warp; k < K; k += kBlock / 32) {
+    double acc = 0.0;
+    for (int b0 = lane; b0 < G; b0 += 32 * kAhead) {
+      double q[kAhead];
 #pragma unroll
-  for (int k = 0; k < K; ++k) acc[k] = 0.0;
-  // The first kRounds rounds of partials (all of them up to kRounds x the block
-  // size) are loaded before any is added, so their L2 latencies overlap; a
-  // round past the grid adds an exact zero, so the sums are those of the plain
-  // loop, in the same order.
-  constexpr int kRounds = 3;
-  {
-    double q[kRounds][K];
+      for (int j = 0; j < kAhead; ++j)
+        if (b0 + 32 * j < G) q[j] = __ldcg(partials + (size_t)(b0 + 32 * j) * kMaxDots + k);
+      if (b0 == lane) acc = q[0];
+      else acc += q[0];
 #pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-      const int b = threadIdx.x + r * blockDim.x;
-#pragma unroll
-      for (int k = 0; k < K; ++k) q[r][k] = b < (int)gridDim.x ? __ldcg(partials + (size_t)b * kMaxDots + k) : 0.0;
+      for (int j = 1; j < kAhead; ++j)
+        if (b0 + 32 * j < G) acc += q[j];
     }
 #pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-#pragma unroll
-      for (int k = 0; k < K; ++k) acc[k] += q[r][k];
-    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) res[k] = acc;
   }
-  for (int b = threadIdx.x + kRounds * blockDim.x; b < (int)gridDim.x; b += blockDim.x) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) acc[k] += __ldcg(partials + (size_t)b * kMaxDots + k);
-  }
-  __shared__ double sm[kBlock / 32][K > 0 ? K : 1];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  {
-    constexpr int P = K <= 1 ? 1 : (K <= 2 ? 2 : (K <= 4 ? 4 : (K <= 8 ? 8 : (K <= 16 ? 16 : 32))));
-    int idx;
-    const double x = warp_sum_multi<K>(acc, idx);
-    if ((lane & (32 / P - 1)) == 0 && idx < K) sm[warp][idx] = x;
-  }
-  __syncthreads();
-  cross_warp_sum<K, kBlock / 32>(sm, res);
   if (threadIdx.x == 0) *counter = 0u;
   __syncthreads();
 }

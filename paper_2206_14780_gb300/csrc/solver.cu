@@ -89,8 +89,8 @@ __global__ void __launch_bounds__(kBlock) k_pass_init(const double* __restrict__
 __global__ void __launch_bounds__(kBlock) k_p_update(int64_t n_pad, Vecs V, const SolverScalars* __restrict__ S) {
   griddep_wait();
   if (S->done) return;
-  const float b0 = (float)S->beta[0], b1 = (float)S->beta[1], b2 = (float)S->beta[2];
-  const float a0 = (float)S->alpha_p[0], a1 = (float)S->alpha_p[1], a2 = (float)S->alpha_p[2];
+  const float b0 = S->beta_f[0], b1 = S->beta_f[1], b2 = S->beta_f[2];
+  const float a0 = S->alphap_f[0], a1 = S->alphap_f[1], a2 = S->alphap_f[2];
   const bool useP = (b0 != 0.f) || (b1 != 0.f) || (b2 != 0.f);
   const bool useA = (a0 != 0.f) || (a1 != 0.f) || (a2 != 0.f);
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_pad; s += (int64_t)gridDim.x * blockDim.x) {
@@ -555,7 +555,7 @@ namespace {
 __global__ void __launch_bounds__(kBlock) k_rstar(int64_t n_pad, Vecs V, const SolverScalars* __restrict__ S) {
   griddep_wait();
   if (S->done) return;
-  const float a0 = (float)S->alpha[0], a1 = (float)S->alpha[1], a2 = (float)S->alpha[2];
+  const float a0 = S->alpha_f[0], a1 = S->alpha_f[1], a2 = S->alpha_f[2];
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_pad; s += (int64_t)gridDim.x * blockDim.x) {
     const float4 r = V.r[s], ap = V.Ap[s];
     V.rs[s] = make_float4(fmaf(-a0, ap.x, r.x), fmaf(-a1, ap.y, r.y), fmaf(-a2, ap.z, r.z), 0.f);
@@ -567,8 +567,8 @@ __global__ void __launch_bounds__(kBlock) k_xr_update(int64_t n_pad, Vecs V, Sol
                                                       unsigned int* counter) {
   griddep_wait();
   if (S->done) return;
-  const float w0 = (float)S->omega[0], w1 = (float)S->omega[1], w2 = (float)S->omega[2];
-  const float al0 = (float)S->alpha[0], al1 = (float)S->alpha[1], al2 = (float)S->alpha[2];
+  const float w0 = S->omega_f[0], w1 = S->omega_f[1], w2 = S->omega_f[2];
+  const float al0 = S->alpha_f[0], al1 = S->alpha_f[1], al2 = S->alpha_f[2];
   float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_pad; s += (int64_t)gridDim.x * blockDim.x) {
     const float4 rs = V.rs[s], as = V.As[s], h = V.rh[s], p = V.p[s];
@@ -602,10 +602,10 @@ __global__ void __launch_bounds__(kBlock) k_xrp_update(int64_t n_pad, Vecs V, So
                                                        unsigned int* counter) {
   griddep_wait();
   if (S->pad) return;
-  const float w0 = (float)S->omega[0], w1 = (float)S->omega[1], w2 = (float)S->omega[2];
-  const float b0 = (float)S->beta[0], b1 = (float)S->beta[1], b2 = (float)S->beta[2];
-  const float a0 = (float)S->alpha_p[0], a1 = (float)S->alpha_p[1], a2 = (float)S->alpha_p[2];
-  const float al0 = (float)S->alpha[0], al1 = (float)S->alpha[1], al2 = (float)S->alpha[2];
+  const float w0 = S->omega_f[0], w1 = S->omega_f[1], w2 = S->omega_f[2];
+  const float b0 = S->beta_f[0], b1 = S->beta_f[1], b2 = S->beta_f[2];
+  const float a0 = S->alphap_f[0], a1 = S->alphap_f[1], a2 = S->alphap_f[2];
+  const float al0 = S->alpha_f[0], al1 = S->alpha_f[1], al2 = S->alpha_f[2];
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_pad; s += (int64_t)gridDim.x * blockDim.x) {
     const float4 rs = V.rs[s], as = V.As[s], p = V.p[s], ap = V.Ap[s];
     float4 d = V.d[s];
@@ -662,7 +662,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_p(int64_t n_pad, Vecs V, const fl
                                                  const SolverScalars* __restrict__ S) {
   griddep_wait();
   if (S->done) return;
-  const float b0 = (float)S->beta[0], b1 = (float)S->beta[1], b2 = (float)S->beta[2];
+  const float b0 = S->beta_f[0], b1 = S->beta_f[1], b2 = S->beta_f[2];
   const bool useP = (b0 != 0.f) || (b1 != 0.f) || (b2 != 0.f);
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_pad; s += (int64_t)gridDim.x * blockDim.x) {
     const float4 r = V.r[s];
@@ -683,7 +683,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_xr(int64_t n_pad, Vecs V, const f
                                                   SolverScalars* S, double* partials, unsigned int* counter) {
   griddep_wait();
   if (S->done) return;
-  const float a0 = (float)S->alpha[0], a1 = (float)S->alpha[1], a2 = (float)S->alpha[2];
+  const float a0 = S->alpha_f[0], a1 = S->alpha_f[1], a2 = S->alpha_f[2];
   float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_pad; s += (int64_t)gridDim.x * blockDim.x) {
     const float4 ap = V.Ap[s], p = V.p[s];

@@ -133,6 +133,9 @@ struct SolverScalars {
   int32_t nonfinite;   // a scalar went NaN/Inf
   int32_t pad;
   int32_t fault;       // an apply kernel gave up a bounded wait (SPH_ERR_TIMEOUT)
+  // float32 copies for the vector updates, made once by the scalar step: a float64
+  // conversion costs a warp 63 cycles, and every warp of those kernels reads them
+  float alpha_f[3], alphap_f[3], beta_f[3], omega_f[3];
   int32_t pad2;
 };
 
