@@ -105,6 +105,37 @@ def test_gradient_over_many_tiles_matches_oracle_and_repeats_exactly(m):
     net.close()
 
 
+@pytest.mark.parametrize("m", [1, 77, 304 * 128 + 128, 2 * 304 * 128 + 1, 4 * 304 * 128 - 60])
+def test_gradient_at_tile_and_buffer_edges(m):
+    """Rows within one tile, and CTAs that walk two, three and four tiles (features and
+    output deltas swap buffers per tile, a tile's last weight gradient runs with the next
+    tile's first product).  Against the oracle with the same bf16 rounding points; what
+    differs is float32 accumulation order and the sigmoid's ~2e-7, so the bounds of the
+    other gradient tests hold."""
+    torch = torch_cuda()
+    from paper_2206_14780_gb300 import binding
+
+    p, X, T, mask = _problem(m=m, seed=11)
+    mask[0] = 1
+    theta = omlp.flatten(p).astype(np.float32)
+    net = binding.Mlp(theta)
+    xb, tt, mk = _dev(torch, X, T, mask)
+    g = torch.empty(binding.MLP_NPARAMS, dtype=torch.float32, device="cuda")
+    loss = torch.empty(1, dtype=torch.float32, device="cuda")
+    net.grad(xb, tt, mk, int(mask.sum()), g, loss)
+    torch.cuda.synchronize()
+    l_ref, g_ref, _ = omlp.loss_and_grad(omlp.unflatten(theta.astype(np.float64)), X, T, mask, bf16=True)
+    gg = g.cpu().numpy().astype(np.float64)
+    assert abs(float(loss.item()) - l_ref) <= 1e-4 * l_ref
+    off = 0
+    for name, shp in omlp.SHAPES:
+        k = int(np.prod(shp))
+        blk, ref = gg[off:off + k], omlp.flatten(g_ref)[off:off + k]
+        assert np.linalg.norm(blk - ref) <= 2e-3 * np.linalg.norm(ref) + 1e-7, name
+        off += k
+    net.close()
+
+
 def test_training_reduces_loss():
     torch = torch_cuda()
     from paper_2206_14780_gb300 import binding
