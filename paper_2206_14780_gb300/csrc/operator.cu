@@ -73,7 +73,7 @@ __global__ void k_op_count(const uint8_t* __restrict__ type, const int32_t* __re
 // Coefficients of A(dt) (Eq. kab with |F|, Eqs. diag, offdiag and dummyvel) in
 // double-float arithmetic (relative error a few 2^-45), stored as the float32
 // pair (hi, lo) that the float32 apply and the double-float residual read;
-// float64 is used once per row (R_b, D) only, and for the Gaussian's exponential.
+// float64 is used once per row (R_b, D) only.
 //   fluid row b:  a_ba = dt c_ab = R_b V_a mubar k(q), D_b = 1 + sum a, with
 //                 Wendland  k = (2 - q)^3,  R_b = 2 dt (105 / (128 pi)) / (h^5 rho_b)
 //                 Gaussian  k = e^{-q^2},   R_b = 2 dt (2 / w_G) / (h^5 rho_b)
@@ -92,6 +92,8 @@ __global__ void k_op_fill(const float4* __restrict__ pos, const float* __restric
     g.periodic[ax] = g64.periodic[ax];
   }
   g.inv_h = df_from_double(g64.inv_h);
+  g.inv_h2 = df_from_double(g64.inv_h * g64.inv_h);
+  const dfl tail = df_from_double(gauss_tail);
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_pad; s += (int64_t)gridDim.x * blockDim.x) {
     if (s >= n || kind[s] == KIND_IDENTITY) {
       invD[s] = 1.f;
@@ -113,8 +115,7 @@ __global__ void k_op_fill(const float4* __restrict__ pos, const float* __restric
         const int32_t t = nbr[base + (int64_t)j * kSlice];
         const float4 pa = pos[t];
         const float4 at = aux[t];
-        const dfl q = df_mul(pair_r_df(pa, pb, g), g.inv_h);
-        const dfl tq3 = fluid_kernel_df(q, gauss);
+        const dfl tq3 = fluid_kernel_df(pair_r2_df(pa, pb, g), g, gauss);
         dfl mub{mu_b, 0.f};
         if (type[t] == SPH_FLUID) {
           if (mean == SPH_MEAN_ARITHMETIC) {
@@ -140,7 +141,7 @@ __global__ void k_op_fill(const float4* __restrict__ pos, const float* __restric
       for (int j = 0; j < c; ++j) {
         const int32_t t = nbr[base + (int64_t)j * kSlice];
         if (type[t] != SPH_FLUID) continue;
-        S = df_add(S, shepard_w_df(df_mul(pair_r_df(pos[t], pb, g), g.inv_h), gauss, gauss_tail));
+        S = df_add(S, shepard_w_df(pair_r2_df(pos[t], pb, g), g, gauss, tail));
       }
       // S rounds to zero only if every fluid neighbour sits at q = 2 to within
       // rounding: zero coefficients then make the row an identity row (as an
@@ -149,7 +150,7 @@ __global__ void k_op_fill(const float4* __restrict__ pos, const float* __restric
       for (int j = 0; j < c; ++j) {
         const int32_t t = nbr[base + (int64_t)j * kSlice];
         if (type[t] != SPH_FLUID) continue;
-        const dfl a = df_mul(shepard_w_df(df_mul(pair_r_df(pos[t], pb, g), g.inv_h), gauss, gauss_tail), invS);
+        const dfl a = df_mul(shepard_w_df(pair_r2_df(pos[t], pb, g), g, gauss, tail), invS);
         const int64_t e = obase + (int64_t)o * kSlice;
         op_ih[e] = make_int2(t, __float_as_int(a.hi));
         op_lo[e] = a.lo;

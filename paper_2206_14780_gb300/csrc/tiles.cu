@@ -55,7 +55,7 @@ struct FillArgs {
   OpGeomDF g;
   dfl kf;              // 2 dt times the constant of |f| over h^5
   int dummy, arithmetic, gauss;
-  double gauss_tail;
+  dfl gauss_tail;      // e^{-9}
   float* hi;
   float* lo;
   int32_t* op_cnt;
@@ -124,8 +124,7 @@ __global__ void __launch_bounds__(256) k_tile_fill(TileView op, FillArgs A) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const float4 pa = tile_at(P, o[k]), at = tile_at(B, o[k]);
-          const dfl q = df_mul(pair_r_df(pa, pb, A.g), A.g.inv_h);
-          const dfl tq3 = fluid_kernel_df(q, A.gauss);
+          const dfl tq3 = fluid_kernel_df(pair_r2_df(pa, pb, A.g), A.g, A.gauss);
           dfl mub{mu_b, 0.f};
           if (pa.w != 0.f) {
             if (A.arithmetic) {
@@ -152,8 +151,7 @@ __global__ void __launch_bounds__(256) k_tile_fill(TileView op, FillArgs A) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           if (g * 4 + k < c)
-            sum = df_add(sum, shepard_w_df(df_mul(pair_r_df(tile_at(P, o[k]), pb, A.g), A.g.inv_h), A.gauss,
-                                           A.gauss_tail));
+            sum = df_add(sum, shepard_w_df(pair_r2_df(tile_at(P, o[k]), pb, A.g), A.g, A.gauss, A.gauss_tail));
       }
     }
     double tot = df_to_double(sum);
@@ -175,7 +173,7 @@ __global__ void __launch_bounds__(256) k_tile_fill(TileView op, FillArgs A) {
         float h4[4], l4[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          dfl a = df_mul(shepard_w_df(df_mul(pair_r_df(tile_at(P, o[k]), pb, A.g), A.g.inv_h), A.gauss, A.gauss_tail),
+          dfl a = df_mul(shepard_w_df(pair_r2_df(tile_at(P, o[k]), pb, A.g), A.g, A.gauss, A.gauss_tail),
                          invS);
           if (g * 4 + k >= c) a = dfl{0.f, 0.f};
           h4[k] = a.hi;
@@ -411,6 +409,7 @@ sph_status tile_fill(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st
   }
   const double ih = 1.0 / (double)H->h;
   A.g.inv_h = split(ih);
+  A.g.inv_h2 = split(ih * ih);
   A.gauss = H->kernel == SPH_KERNEL_GAUSSIAN ? 1 : 0;
   A.kf = split(2.0 * P->dt * (A.gauss ? 2.0 / gauss_norm() : 105.0 / (128.0 * M_PI)) * (ih * ih * ih * ih * ih));
   A.pos = H->pos_s.p;
@@ -422,7 +421,7 @@ sph_status tile_fill(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st
   A.n = H->n;
   A.dummy = P->boundary == SPH_BC_DUMMY ? 1 : 0;
   A.arithmetic = P->mean == SPH_MEAN_ARITHMETIC ? 1 : 0;
-  A.gauss_tail = std::exp(-kGaussK * kGaussK);
+  A.gauss_tail = split(std::exp(-kGaussK * kGaussK));
   A.hi = H->t_hi.p;
   A.lo = H->t_lo.p;
   A.op_cnt = H->op_cnt.p;

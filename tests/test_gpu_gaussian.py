@@ -99,3 +99,29 @@ def test_gaussian_rejections_and_capacity():
     feats = torch.empty((s.n, 16), dtype=torch.int16, device="cuda")
     binding.mlp_features(nb, params_for(s), v, feats)
     net.close()
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("name", sorted(GAUSS_SCENES))
+def test_gaussian_coefficients_to_float64_accuracy(name, form):
+    """The residual b - A x in the tile form and, after a solve forced onto the SELL-32
+    rows (form 1), the solution at 1e-9: e^{-q^2} in double-float (2^-43 a pair at most)
+    leaves coefficients good to a few 2^-45 in the mean, so the residual is within 1e-12
+    of ||b|| + |||A| |x||| and a 1e-9 residual by A's own coefficients is one by the
+    oracle's."""
+    torch = torch_cuda()
+    from paper_2206_14780_gb300 import binding
+
+    s = GAUSS_SCENES[name]()
+    nb, _ = lib_build(s, max_neighbors=MAXNB)
+    _, _, A = oracle_system(s)
+    if form == 0:
+        x = np.random.default_rng(8).normal(size=(s.n, 3))
+        rt = torch.empty((s.n, 3), dtype=torch.float64, device="cuda")
+        nb.residual(params_for(s), torch.from_numpy(x).cuda(), torch.from_numpy(s.b).cuda(), rt)
+        scale = np.linalg.norm(s.b) + np.linalg.norm(abs(A) @ abs(x))
+        assert np.linalg.norm(rt.cpu().numpy() - (s.b - A @ x)) < 1e-12 * scale
+    else:
+        x, rep = gpu_solve(nb, s, binding.solve_opts(rtol=1e-9, apply_form=1))
+        assert rep["status"] == 0, rep
+        assert oop.true_residual(A, x, s.b)[0] <= 1.1e-9
