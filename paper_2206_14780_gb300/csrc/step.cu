@@ -92,15 +92,38 @@ __device__ __forceinline__ float kernel_w(float q, const StepGeom& g) {
   return g.w_scale * t2 * t2 * fmaf(2.f, q, 1.f);
 }
 
-__device__ __forceinline__ double eos_d(double rho, double rho0, double c0, double zeta) {
-  return c0 * c0 * rho0 / zeta * (pow(rho / rho0, zeta) - 1.0);
+// The equation of state's exponent: zeta itself, and k = zeta where that is a whole
+// number from 2 to 16 (7 for water), else 0.  A float64 instruction costs a warp ~63
+// cycles and pow over a hundred of them; x^k by squaring is 4 at k = 7, and the root one
+// Halley step from the float32 root (error (k^2 - 1) / 12 e^3 of its ~3e-7), both within
+// a few units of float64's last place before the result is rounded to float32.
+struct Zeta {
+  double z;
+  int k;
+};
+Zeta make_zeta(double z) { return Zeta{z, z >= 2.0 && z <= 16.0 && z == std::floor(z) ? (int)z : 0}; }
+
+__device__ __forceinline__ double whole_pow(double x, int k) {
+  double r = (k & 1) ? x : 1.0;
+  for (k >>= 1; k > 0; k >>= 1) {
+    x *= x;
+    if (k & 1) r *= x;
+  }
+  return r;
+}
+__device__ __forceinline__ double zeta_pow(double x, Zeta e) { return e.k ? whole_pow(x, e.k) : pow(x, e.z); }
+__device__ __forceinline__ double zeta_root(double v, Zeta e) {
+  if (e.k == 0 || !(v > 1e-30 && v < 1e30)) return pow(v, 1.0 / e.z);
+  const double y = (double)powf((float)v, 1.f / (float)e.k), p = whole_pow(y, e.k);
+  return y + y * (2.0 * (v - p)) / ((double)(e.k + 1) * p + (double)(e.k - 1) * v);
 }
 
 // P = EOS(rho) on every sorted row (dummy walls are overwritten by the closure)
-__global__ void k_step_eos(const float* __restrict__ rho_s, int64_t n, double rho0, double c0, double zeta,
+__global__ void k_step_eos(const float* __restrict__ rho_s, int64_t n, double rho0, double c0, Zeta zeta,
                            float* __restrict__ P_s) {
+  const double scale = c0 * c0 * rho0 / zeta.z;
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x)
-    P_s[s] = (float)eos_d((double)rho_s[s], rho0, c0, zeta);
+    P_s[s] = (float)(scale * (zeta_pow((double)rho_s[s] / rho0, zeta) - 1.0));
 }
 
 // dummy walls (Eq. dummyP): pressure from the fluid neighbours, density by the
@@ -109,7 +132,7 @@ __global__ void k_step_dummy(const float4* __restrict__ pos_s, float* __restrict
                              const uint8_t* __restrict__ type_s, const int32_t* __restrict__ cnt,
                              const int64_t* __restrict__ slice_off, const int32_t* __restrict__ nbr,
                              const int32_t* __restrict__ perm, int64_t n, StepGeom g, double gx, double gy, double gz,
-                             double rho0, double c0, double zeta, float* __restrict__ P_s, float* __restrict__ rho_c) {
+                             double rho0, double c0, Zeta zeta, float* __restrict__ P_s, float* __restrict__ rho_c) {
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
     if (type_s[s] == SPH_FLUID) continue;
     const float4 pb = pos_s[s];
@@ -129,7 +152,7 @@ __global__ void k_step_dummy(const float4* __restrict__ pos_s, float* __restrict
       num += w * ((double)P_s[t] + gr * (double)rho_s[t]);
     }
     const double P = S > 0.0 ? num / S : 0.0;
-    const double r = rho0 * pow(P * zeta / (c0 * c0 * rho0) + 1.0, 1.0 / zeta);
+    const double r = rho0 * zeta_root(P * zeta.z / (c0 * c0 * rho0) + 1.0, zeta);
     P_s[s] = (float)P;
     rho_s[s] = (float)r;
     rho_c[perm[s]] = (float)r;
@@ -223,7 +246,7 @@ template <int TS>
 __global__ void __launch_bounds__(256) k_tile_dummy(TileLists L, const float4* __restrict__ pos_s, float* rho_s,
                                                     const uint8_t* __restrict__ type_s, const int32_t* __restrict__ perm,
                                                     int64_t n, StepGeom g, dfl gx, dfl gy, dfl gz, double rho0, double c0,
-                                                    double zeta, float* P_s, float* __restrict__ rho_c) {
+                                                    Zeta zeta, float* P_s, float* __restrict__ rho_c) {
   constexpr int S = 8 / TS, R = 32 * TS;
   extern __shared__ __align__(16) float4 dyn[];
   __shared__ float part[S > 1 ? S - 1 : 1][4][R];
@@ -274,7 +297,7 @@ __global__ void __launch_bounds__(256) k_tile_dummy(TileLists L, const float4* _
     if (wall && split == 0) {
       const double Sw = W.value();
       const double P = Sw > 0.0 ? df_to_double(num) / Sw : 0.0;
-      const double r = rho0 * pow(P * zeta / (c0 * c0 * rho0) + 1.0, 1.0 / zeta);
+      const double r = rho0 * zeta_root(P * zeta.z / (c0 * c0 * rho0) + 1.0, zeta);
       P_s[s] = (float)P;
       rho_s[s] = (float)r;
       rho_c[perm[s]] = (float)r;
@@ -501,8 +524,9 @@ sph_status evaluate(sph_state* S, const sph_step_params* Pp, sph_neighbors** han
     SPH_TRY(mu_papanastasiou(H, S->vel, S->vel, Pp->tau0, Pp->mu0, Pp->m, S->mu, 1, st));
   if (!H->tile_ok) SPH_TRY(ensure_nbr(H, st));
   const StepGeom g = step_geom(H, S);
+  const Zeta zeta = make_zeta(Pp->zeta);
   const int grid = grid_for(H, H->n);
-  SPH_LAUNCH(k_step_eos, grid, kBlock, 0, st)(H->rho_s.p, H->n, Pp->rho0, Pp->c0, Pp->zeta, T.P_s.p);
+  SPH_LAUNCH(k_step_eos, grid, kBlock, 0, st)(H->rho_s.p, H->n, Pp->rho0, Pp->c0, zeta, T.P_s.p);
   const int dummy = Pp->boundary == SPH_BC_DUMMY ? 1 : 0;
   const float4* vel = reinterpret_cast<const float4*>(S->vel);
   const size_t smem = tile_smem(H, 32);
@@ -515,11 +539,11 @@ sph_status evaluate(sph_state* S, const sph_step_params* Pp, sph_neighbors** han
       auto kern = SPH_TILE_PICK(H, k_tile_dummy);
       SPH_LAUNCH(kern, tile_grid(H, (const void*)kern, smem), 256, smem, st)(
           tile_lists(H), H->pos_s.p, H->rho_s.p, H->type_s.p, H->perm.p, H->n, g, split(Pp->g[0]), split(Pp->g[1]),
-          split(Pp->g[2]), Pp->rho0, Pp->c0, Pp->zeta, T.P_s.p, S->rho);
+          split(Pp->g[2]), Pp->rho0, Pp->c0, zeta, T.P_s.p, S->rho);
     } else {
       SPH_LAUNCH(k_step_dummy, grid, kBlock, 0, st)(H->pos_s.p, H->rho_s.p, H->type_s.p, H->cnt.p, H->slice_off.p,
                                                      H->nbr.p, H->perm.p, H->n, g, Pp->g[0], Pp->g[1], Pp->g[2],
-                                                     Pp->rho0, Pp->c0, Pp->zeta, T.P_s.p, S->rho);
+                                                     Pp->rho0, Pp->c0, zeta, T.P_s.p, S->rho);
     }
     H->mu_version++;   // the walls' densities enter A(dt): set it up again
   }

@@ -91,6 +91,27 @@ def test_one_step_matches_oracle(name):
         np.testing.assert_allclose(mu[fl], info["half"]["mu"][fl].astype(np.float64), rtol=1e-4)
 
 
+@pytest.mark.parametrize("zeta", [1.0, 2.0, 6.5, 16.0, 17.0])
+def test_equation_of_state_exponents_match_oracle(zeta):
+    """Exponents on both sides of the whole-number path (2 to 16): pressures and the walls'
+    inverse, which the step's densities and velocities follow.  Bounds as in
+    test_one_step_matches_oracle: the exponent's path changes nothing above float64
+    rounding."""
+    from paper_2206_14780_gb300 import binding
+
+    make, prm = STEP_CASES["couette_dummy"]
+    s, prm = make(), dict(prm, zeta=zeta)
+    st, t = _stepper(s)
+    rep = st.step(_params(s, prm), binding.solve_opts(rtol=1e-10, eps_inner=1e-3))
+    st.close()
+    assert rep["status"] == 0, rep
+    new, info = ostep.step(s, prm)
+    fl = s.ptype == scenes.FLUID
+    u = t["vel"].cpu().numpy()[:, :3].astype(np.float64)
+    assert np.linalg.norm(u[fl] - info["u_new"][fl]) < 1e-5 * np.linalg.norm(info["u_new"][fl])
+    np.testing.assert_allclose(t["rho"].cpu().numpy().astype(np.float64), new.rho.astype(np.float64), rtol=2e-6)
+
+
 def test_fluid_at_rest_stays_at_rest_on_the_gpu():
     from paper_2206_14780_gb300 import binding
 
