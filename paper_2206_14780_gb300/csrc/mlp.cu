@@ -71,30 +71,46 @@ __global__ void k_mlp_pack(const float* __restrict__ th, MlpPack* __restrict__ P
 
 // grad[i] = sum over the partial gradients of the nblocks training CTAs; loss = sum of
 // their losses * inv_cnt.  One block per 32 parameters: warp g sums the partials
-// g, g + 8, g + 16, ... in order, then the eight warp sums are added in warp order,
-// so the result does not depend on the run.
+// g, g + 8, g + 16, ... in order, then the eight warp sums are added in warp order; one
+// more block sums the losses over the lanes of a warp, so the results do not depend on
+// the run.  Bound by load latency: eight of a warp's partials are in flight at once.
+// Each result also goes to the caller's array where there is one.
 constexpr int kReduceWarps = 8;
+constexpr int kReduceBlocks = (kNP + 31) / 32 + 1;
 __global__ void __launch_bounds__(kReduceWarps * 32)
     k_mlp_reduce(const float* __restrict__ partial, const float* __restrict__ loss_part, int nblocks, float inv_cnt,
-                 float* __restrict__ grad, float* __restrict__ loss) {
+                 float* __restrict__ grad, float* __restrict__ loss, float* __restrict__ grad_out,
+                 float* __restrict__ loss_out) {
   __shared__ float part[kReduceWarps][32];
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  if (blockIdx.x == kReduceBlocks - 1) {
+    if (g > 0) return;
+    float t = 0.f;
+    for (int b = lane; b < nblocks; b += 32) t += loss_part[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) {
+      *loss = t * inv_cnt;
+      if (loss_out) *loss_out = t * inv_cnt;
+    }
+    return;
+  }
   const int i = blockIdx.x * 32 + lane;
   float s = 0.f;
-  if (i < kNP)
+  if (i < kNP) {
+#pragma unroll 8
     for (int b = g; b < nblocks; b += kReduceWarps) s += partial[(size_t)b * kNP + i];
+  }
   part[g][lane] = s;
   __syncthreads();
   if (g == 0) {
     float t = 0.f;
 #pragma unroll
     for (int w = 0; w < kReduceWarps; ++w) t += part[w][lane];
-    if (i < kNP) grad[i] = t;
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 32) {
-    float t = 0.f;
-    for (int b = 0; b < nblocks; ++b) t += loss_part[b];
-    *loss = t * inv_cnt;
+    if (i < kNP) {
+      grad[i] = t;
+      if (grad_out) grad_out[i] = t;
+    }
   }
 }
 
@@ -262,7 +278,7 @@ sph_status sph_mlp_forward(const sph_mlp* M, const uint16_t* feats, int64_t m, f
 }
 
 static sph_status mlp_grad_impl(sph_mlp* M, const uint16_t* feats, const float* targets, const uint8_t* mask,
-                                int64_t m, float inv_cnt, cudaStream_t st) {
+                                int64_t m, float inv_cnt, float* grad_out, float* loss_out, cudaStream_t st) {
   int dev = 0, sms = 0;
   SPH_TRY_CUDA(cudaGetDevice(&dev));
   SPH_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -274,8 +290,8 @@ static sph_status mlp_grad_impl(sph_mlp* M, const uint16_t* feats, const float* 
   float* loss_part = M->partial.p + (size_t)blocks * kNP;
   SPH_TRY(mlp_grad_tc(M, reinterpret_cast<const __nv_bfloat16*>(feats), reinterpret_cast<const float4*>(targets),
                       mask, m, inv_cnt, M->partial.p, loss_part, M->fault.p, (int)blocks, st));
-  SPH_LAUNCH(k_mlp_reduce, (kNP + 31) / 32, kReduceWarps * 32, 0, st)(M->partial.p, loss_part, (int)blocks, inv_cnt,
-                                                                      M->grad.p, M->loss.p);
+  SPH_LAUNCH(k_mlp_reduce, kReduceBlocks, kReduceWarps * 32, 0, st)(M->partial.p, loss_part, (int)blocks, inv_cnt,
+                                                                    M->grad.p, M->loss.p, grad_out, loss_out);
   SPH_TRY_CUDA(cudaGetLastError());
   return SPH_OK;
 }
@@ -288,10 +304,7 @@ sph_status sph_mlp_grad(sph_mlp* M, const uint16_t* feats, const float* targets,
     return SPH_ERR_INVALID;
   }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  SPH_TRY(mlp_grad_impl(M, feats, targets, mask, m, 1.f / (float)count, st));
-  if (grad_out) SPH_TRY_CUDA(cudaMemcpyAsync(grad_out, M->grad.p, kNP * 4, cudaMemcpyDeviceToDevice, st));
-  if (loss_out) SPH_TRY_CUDA(cudaMemcpyAsync(loss_out, M->loss.p, 4, cudaMemcpyDeviceToDevice, st));
-  return SPH_OK;
+  return mlp_grad_impl(M, feats, targets, mask, m, 1.f / (float)count, grad_out, loss_out, st);
 }
 
 sph_status sph_mlp_train_step(sph_mlp* M, const uint16_t* feats, const float* targets, const uint8_t* mask,
@@ -302,7 +315,7 @@ sph_status sph_mlp_train_step(sph_mlp* M, const uint16_t* feats, const float* ta
     return SPH_ERR_INVALID;
   }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  SPH_TRY(mlp_grad_impl(M, feats, targets, mask, m, 1.f / (float)count, st));
+  SPH_TRY(mlp_grad_impl(M, feats, targets, mask, m, 1.f / (float)count, nullptr, nullptr, st));
   M->step += 1;
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   const float c1 = 1.f - std::pow(b1, (float)M->step), c2 = 1.f - std::pow(b2, (float)M->step);
