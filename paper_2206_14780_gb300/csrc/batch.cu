@@ -167,7 +167,7 @@ __device__ __forceinline__ void tile_rows(const BatchView& B, int t, int64_t& fi
 
 // ---- the tile form inside a batch tile -----------------------------------------------
 // A batch tile of a scene is a run of that scene's tiles (16, 32 and 64 slices are
-// whole numbers of 2, 4 or 8): the block takes them one after the other, each with its
+// whole numbers of 1, 2, 4 or 8): the block takes them one after the other, each with its
 // union in shared memory and 8 / ts threads per row.
 struct TileLane {
   int split, splits, row, rows;   // the thread's share of a row and its row in the tile
@@ -188,7 +188,7 @@ __device__ __forceinline__ TileLane tile_lane(const SceneDesc& d, int64_t tile) 
 }
 
 // fin(row, v_b, y) for the rows of batch tile [sl0, sl0 + nsl) of y = D^-1 A v; u: the
-// union, part: [3][64][3] floats
+// union, part: [7][32][3] floats, the most any ts takes
 template <class Fin>
 __device__ __forceinline__ void batch_apply(const SceneDesc& d, const float4* __restrict__ v, int64_t sl0, int nsl,
                                             float4* u, float* part, Fin fin) {
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kBlock) kb_split(BatchView B, int64_t nrows) {
 template <bool TILE>
 __global__ void __launch_bounds__(kBlock) kb_residual(BatchView B) {
   extern __shared__ __align__(16) float4 dyn[];
-  __shared__ double rpart[TILE ? 192 * 3 : 1];
+  __shared__ double rpart[TILE ? 224 * 3 : 1];
   if (threadIdx.x == 0 && blockIdx.x == 0) {   // counted by kb_init
     B.ctrl->active = 0;
     B.ctrl->passes += 1;
@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(kBlock) kb_init(BatchView B) {
 template <int U, bool PF, int NB, bool TILE>
 __global__ void __launch_bounds__(NB, TILE ? 4 : 1) kb_pass(BatchView B, int iter_cap) {
   extern __shared__ __align__(16) float4 dyn[];
-  __shared__ float part[TILE ? 192 * 3 : 1];
+  __shared__ float part[TILE ? 224 * 3 : 1];
   for (int it = 0; it < iter_cap; ++it) {
     if (*(volatile int32_t*)&B.ctrl->active == 0) break;
     // phase 1: p = r + beta p - alpha' Ap

@@ -691,8 +691,8 @@ __global__ void __launch_bounds__(256) k_tile_plan(const uint8_t* __restrict__ t
   constexpr int R = 32 * TS, S = 8 / TS;
   extern __shared__ __align__(16) uint16_t dyn[];
   uint16_t* list = dyn;                                        // [maxnb][R]
-  uint16_t* map = list + (size_t)maxnb * R;                    // [cap]
-  uint8_t* mark = reinterpret_cast<uint8_t*>(map + cap);       // [cap]: 1 referenced, 2 wall
+  uint16_t* map = list + (size_t)maxnb * R;                    // [cap]: place | kRef | kWall
+  constexpr unsigned kRef = 0x4000u, kWall = 0x8000u;
   __shared__ int wpre[256];
   __shared__ int wsum[8];
   if (build_stopped(flags, maxnb) || (flags[0] & (FLAG_REGION | FLAG_CAPACITY)) != 0) return;
@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(256) k_tile_plan(const uint8_t* __restrict__ t
     const int2 a = cells[c];
     const int off = a.y & 0xffff, many = a.y >> 16, padded = (many + 3) & ~3;
     for (int k = lane; k < padded; k += 32)
-      mark[off + k] = k < many && type_s[a.x + k] != SPH_FLUID ? 2 : 0;
+      map[off + k] = k < many && type_s[a.x + k] != SPH_FLUID ? kWall : 0;
   }
   __syncthreads();
   const int row = tid % R, split = tid / R, rl = row & 31;
@@ -713,15 +713,16 @@ __global__ void __launch_bounds__(256) k_tile_plan(const uint8_t* __restrict__ t
   const int c = live ? cnt[s] : 0;
   const uint16_t* __restrict__ mine = raw + (s / kSlice) * (int64_t)(kSlice * maxnb) + rl;
 #pragma unroll 4
-  for (int j = split; j < c; j += S) mark[mine[j * kSlice]] |= 1;
+  for (int j = split; j < c; j += S) map[mine[j * kSlice]] |= kRef;
   __syncthreads();
   // positions: word w covers region places 32 w .. 32 w + 31
   const int words = (nreg + 31) >> 5;
   for (int w = wid; w < words; w += 8) {
     const int p = w * 32 + lane;
-    const unsigned bl = __ballot_sync(0xffffffffu, p < nreg && (mark[p] & 1));
+    const unsigned f = p < nreg ? map[p] : 0u;
+    const unsigned bl = __ballot_sync(0xffffffffu, (f & kRef) != 0);
     if (lane == 0) wpre[w] = __popc(bl);
-    if (p < nreg) map[p] = (uint16_t)__popc(bl & ((1u << lane) - 1u));
+    if (p < nreg) map[p] = (uint16_t)(f | __popc(bl & ((1u << lane) - 1u)));
   }
   __syncthreads();
   {
@@ -745,22 +746,22 @@ __global__ void __launch_bounds__(256) k_tile_plan(const uint8_t* __restrict__ t
     }
   }
   __syncthreads();
-  // map: union position, 0x8000 on walls (positions stay below 4,096)
+  // map: union position, kWall on walls (positions stay below 4,096)
   for (int q = wid; q < m; q += 8) {
     const int2 a = cells[q];
     const int off = a.y & 0xffff, many = a.y >> 16;
     for (int k = lane; k < many; k += 32) {
       const int p = off + k;
-      const int u = map[p] + wpre[p >> 5];
-      const uint8_t f = mark[p];
-      map[p] = (uint16_t)(u | ((f & 2) ? 0x8000 : 0));
-      if ((f & 1) && u < ustride) uni[tile * ustride + u] = a.x + k;
+      const unsigned f = map[p];
+      const int u = (int)(f & 31u) + wpre[p >> 5];
+      map[p] = (uint16_t)(u | (f & kWall));
+      if ((f & kRef) && u < ustride) uni[tile * ustride + u] = a.x + k;
     }
   }
   __syncthreads();
   if (split > 0 || s >= nslices * kSlice) return;
   const bool fluid = live && type_s[s] == SPH_FLUID;
-  const unsigned skip = fluid ? 0u : 0x8000u;   // entries left out of the interleaving
+  const unsigned skip = fluid ? 0u : kWall;   // entries left out of the interleaving
   Fields<WIDE> left, cur;
   int nf = 0;
 #pragma unroll 4
@@ -971,11 +972,15 @@ sph_status build_slices(sph_neighbors* H, const int32_t* cnt, int64_t* off, int6
   return SPH_OK;
 }
 
-// places in shared memory for a tile's search region; 256-row tiles of the box need
-// up to ~3,100 (2,757 particles and the cells' padding), the Gaussian's narrow channels
-// ~3,600, h = 2.5 dp 6,656
-constexpr int kRegionSmall = 4608;
-constexpr int kRegionLarge = 7168;
+// places in shared memory for a tile's search region, tried in turn: 256-row tiles of the
+// box need up to ~3,100 (2,757 particles and the cells' padding), the Gaussian's narrow
+// channels ~3,600, h = 2.5 dp 6,656.  With the first and 128 entries a row three blocks of
+// the plan fit an SM (72.7 KB each; two with 4,608 places); above 160 entries a row it
+// changes nothing and the second comes first.  A handle starts with the size that its
+// last rebuild needed.
+constexpr int kRegions[] = {3584, 4608, 7168};
+constexpr int kRegionSizes = 3;
+constexpr int kRegionLarge = kRegions[kRegionSizes - 1];
 
 // Slices per tile.  Large tiles share more of their neighbours (4.4 union rows per row
 // at 8 slices, 5.8 at 4, 7.8 at 2 on the box); small ones give a small set more blocks
@@ -985,9 +990,16 @@ constexpr int kRegionLarge = 7168;
 // five-kernel loop: 64k rows 17.3 / 16.5 / 18.0 us, 274k 37.5 / 37.5 / 41.4, 1,157k 128 / 138 / 161.
 // The Gaussian's unions are larger and its rows longer: apply at 190k rows 67.8 / 53.6 /
 // 56.4, but at 77k the cooperative kernel holds 8 slices better (6117 / 7213 us a solve).
+// One slice where that gives fewer tiles than SMs (twice as many with rows of ~250):
+// the set-up kernels' chains per row halve.  Against two slices, us a pass: step of 1.4k
+// rows 890 -> 855, 2.6k 896 -> 812, 4.6k 925 -> 876, solve of 2.7k 1058 -> 990; Gaussian
+// steps of 4.7k, 5.6k, 9.2k rows 1538 -> 1348, 1637 -> 1537, 1367 -> 1214, Gaussian solves
+// 1% either way.  Beyond, two slices are as fast or faster (solve of 6.8k rows 1395 / 1485).
+// 2,400-3,040 slices of ~80 in tiles of 4: 1-10% slower than 8 everywhere.
 // Beyond 320 (640) entries per row the lists of 8 (4) slices exceed the plan's shared
 // memory.
 static int tile_slices_for(int64_t nslices, int32_t maxnb, int num_sms) {
+  if (nslices < (maxnb > 160 ? 2 : 1) * (int64_t)num_sms) return 1;
   if (nslices < 600 || maxnb > 640) return 2;
   if (nslices < 1800 || maxnb > 320) return 4;
   return maxnb > 160 && nslices > 18 * (int64_t)num_sms ? 4 : 8;
@@ -1015,7 +1027,7 @@ template <int TS>
 static sph_status launch_search_ts(sph_neighbors* H, const Grid& g, const BandIn& bin, int32_t maxnb, int cap,
                                    cudaStream_t st) {
   const size_t smem = (size_t)cap * 3 * sizeof(float);
-  const size_t plan = (size_t)maxnb * 32 * TS * sizeof(uint16_t) + (size_t)cap * 3;
+  const size_t plan = (size_t)maxnb * 32 * TS * sizeof(uint16_t) + (size_t)cap * sizeof(uint16_t);
   const bool per = g.periodic[0] || g.periodic[1] || g.periodic[2];
   auto search = per ? k_tile_search<TS, true> : k_tile_search<TS, false>;
   auto planner = maxnb > 255 ? k_tile_plan<TS, true> : k_tile_plan<TS, false>;
@@ -1053,7 +1065,8 @@ static sph_status launch_tile_search(sph_neighbors* H, const Grid& g, const Band
   SPH_TRY_CUDA(cudaMemsetAsync(H->tmp_i32b.p, 0, H->nslices * sizeof(int32_t), st));
   if (ts == 8) SPH_TRY(launch_search_ts<8>(H, g, bin, maxnb, cap, st));
   else if (ts == 4) SPH_TRY(launch_search_ts<4>(H, g, bin, maxnb, cap, st));
-  else SPH_TRY(launch_search_ts<2>(H, g, bin, maxnb, cap, st));
+  else if (ts == 2) SPH_TRY(launch_search_ts<2>(H, g, bin, maxnb, cap, st));
+  else SPH_TRY(launch_search_ts<1>(H, g, bin, maxnb, cap, st));
   return scan<int64_t>(H, H->tmp_i32b.p, H->t_off.p, H->nslices, kSlice, nullptr, st);
 }
 
@@ -1204,13 +1217,13 @@ sph_status build_neighbors(const sph_scene* sc, int32_t maxnb, sph_neighbors** o
   H->tile_ok = false;
   int32_t hflags[8];
   int64_t tot[2], t_entries = 0;
-  // the tile search with a small region first, with a large one for the sets that
+  // the tile search with a small region first, with larger ones for the sets that
   // need it (h = 2.5 dp: 150 particles per cell), then the global scan
-  for (int round = 0;; ++round) {
-    const bool tiles = round < 2;
+  for (int round = std::max(H->region, maxnb > 160 ? 1 : 0);; ++round) {
+    const bool tiles = round < kRegionSizes;
     TRYF_CUDA(cudaMemsetAsync(H->tmp_i64.p, 0, 2 * sizeof(int64_t), st));
     if (tiles) {
-      TRYF(launch_tile_search(H, g, bin, maxnb, round == 0 ? kRegionSmall : kRegionLarge, st));
+      TRYF(launch_tile_search(H, g, bin, maxnb, kRegions[round], st));
       TRYF_CUDA(cudaMemcpyAsync(&t_entries, H->t_off.p + H->nslices, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     } else {
       TRYF_CUDA(cudaMemcpyAsync(hflags, H->flags.p, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -1249,7 +1262,7 @@ sph_status build_neighbors(const sph_scene* sc, int32_t maxnb, sph_neighbors** o
     if (tiles && ((hflags[0] & FLAG_REGION) || hflags[3] > kTileUnion)) {
       TRYF_CUDA(cudaMemsetAsync(H->flags.p, 0, sizeof(int32_t), st));
       TRYF_CUDA(cudaMemsetAsync(H->flags.p + 3, 0, sizeof(int32_t), st));
-      if (hflags[3] > kTileUnion) round = 1;   // a larger region does not help
+      if (hflags[3] > kTileUnion) round = kRegionSizes - 1;   // a larger region does not help
       continue;
     }
     if (hflags[0] & FLAG_CAPACITY) {
@@ -1258,6 +1271,7 @@ sph_status build_neighbors(const sph_scene* sc, int32_t maxnb, sph_neighbors** o
     }
     H->tile_ok = tiles;
     H->nbr_valid = !tiles;
+    H->region = tiles ? round : 0;
     break;
   }
   H->tile_umax = hflags[3];

@@ -537,6 +537,15 @@ PersistPlan persist_plan(const sph_neighbors* H) {
   const int sms = H->num_sms > 0 ? H->num_sms : 1;
   if (!H->op_tile_valid || H->ntiles < 1) return p;
   p.tiles_per_block = (int)((H->ntiles + sms - 1) / sms);
+  // One-slice tiles: fewer blocks with more tiles each, since an exchange costs the more
+  // the more blocks take part.  Whole passes with 1 / 2 / 3 / 4 tiles a block, us: rows of
+  // ~80, solves of 2.7k rows 1133 / 1078 / 990 / 1026, 3.2k from host buffers 816 / 749 /
+  // 760 / 735, a step of 2.6k 842 / 841 / 812 / 838; rows of ~250, 2.9k rows 1079 / 1103 /
+  // 1168 / 1204, 4.7k 1590 / 1430 / 1473 / 1530.
+  if (H->tile_ts == 1) {
+    const int least = H->maxnb <= 160 ? 3 : (H->ntiles <= 2 * (int64_t)sms / 3 ? 1 : 2);
+    p.tiles_per_block = (p.tiles_per_block + least - 1) / least * least;
+  }
   const int nsl = p.tiles_per_block * H->tile_ts;
   if (p.tiles_per_block > kPTilesMax || nsl > kPSliceMax) return p;
   p.grid = (int)((H->ntiles + p.tiles_per_block - 1) / p.tiles_per_block);
@@ -571,7 +580,7 @@ sph_status persist_solve(sph_neighbors* H, const PersistPlan& plan, const TileVi
   SPH_TRY_CUDA(cudaMemsetAsync(H->persist_buf.p, 0, (nslots * 2 + 32) * sizeof(double), st));
   PersistArgs A{};
   A.op = view;
-  A.ts_shift = H->tile_ts == 8 ? 3 : (H->tile_ts == 4 ? 2 : 1);
+  A.ts_shift = H->tile_ts == 8 ? 3 : (H->tile_ts == 4 ? 2 : (H->tile_ts == 2 ? 1 : 0));
   A.tiles_per_block = plan.tiles_per_block;
   A.splits = plan.splits;
   A.ucap = plan.ucap;

@@ -497,7 +497,8 @@ __global__ void __launch_bounds__(256, kTileBlocks) k_tile_apply_dot(TileView op
 using TileDotFn = void (*)(TileView, const float4*, float4*, const float4*, SolverScalars*, double*, unsigned int*);
 template <int PH>
 TileDotFn tile_dot_kernel(int ts) {
-  return ts == 8 ? k_tile_apply_dot<PH, 8> : (ts == 4 ? k_tile_apply_dot<PH, 4> : k_tile_apply_dot<PH, 2>);
+  return ts == 8 ? k_tile_apply_dot<PH, 8>
+                 : (ts == 4 ? k_tile_apply_dot<PH, 4> : (ts == 2 ? k_tile_apply_dot<PH, 2> : k_tile_apply_dot<PH, 1>));
 }
 
 }  // namespace

@@ -203,6 +203,7 @@ struct sph_neighbors {
   int32_t maxnb = 0;               // capacity of the lists
   bool tile_ok = false, nbr_valid = false;
   int tile_ts = 8;                 // slices per tile
+  int region = 0;                  // size class of the search region the last rebuild needed
   int64_t ntiles = 0, t_istride = 0, t_entries = 0;
   int32_t t_ustride = 0, tile_umax = 0;
   sph::DBuf<uint16_t> t_idx;       // [nslices][t_istride] union positions x 16

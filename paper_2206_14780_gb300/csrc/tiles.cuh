@@ -245,9 +245,10 @@ __device__ __forceinline__ void tile_residual_row(const TileView& op, const floa
 TileView tile_view(const sph_neighbors* H);
 // dynamic shared memory of a kernel that holds `bytes_per_row` of every union row
 size_t tile_smem(const sph_neighbors* H, int bytes_per_row);
-// one of a kernel template's three instances, by the handle's slices per tile
-#define SPH_TILE_PICK(H, name, ...) \
-  ((H)->tile_ts == 8 ? name<8 __VA_ARGS__> : ((H)->tile_ts == 4 ? name<4 __VA_ARGS__> : name<2 __VA_ARGS__>))
+// one of a kernel template's four instances, by the handle's slices per tile
+#define SPH_TILE_PICK(H, name, ...)                                                                              \
+  ((H)->tile_ts == 8 ? name<8 __VA_ARGS__>                                                                       \
+                     : ((H)->tile_ts == 4 ? name<4 __VA_ARGS__> : ((H)->tile_ts == 2 ? name<2 __VA_ARGS__> : name<1 __VA_ARGS__>)))
 #define SPH_COMMA ,
 
 // blocks for a tile kernel: every tile, or as many as are resident at once
