@@ -92,6 +92,12 @@ __device__ __forceinline__ dfl df_from_double(double x) {
   const float hi = __double2float_rn(x);
   return dfl{hi, __double2float_rn(x - (double)hi)};
 }
+// a row of x as float32 hi + lo (x = hi + lo to ~2^-48 relative): out[0] hi, out[1] lo
+__device__ __forceinline__ void split_x(const double (&x)[3], float4* out) {
+  const float h0 = (float)x[0], h1 = (float)x[1], h2 = (float)x[2];
+  out[0] = make_float4(h0, h1, h2, 0.f);
+  out[1] = make_float4((float)(x[0] - (double)h0), (float)(x[1] - (double)h1), (float)(x[2] - (double)h2), 0.f);
+}
 __device__ __forceinline__ double df_to_double(dfl a) { return (double)a.hi + (double)a.lo; }
 
 }  // namespace sph

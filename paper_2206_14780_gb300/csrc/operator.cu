@@ -190,13 +190,10 @@ __global__ void k_scatter_f4(const float4* __restrict__ y_s, const int32_t* __re
     reinterpret_cast<float4*>(y_caller)[perm[s]] = y_s[s];
 }
 
-// x64 -> float32 hi + lo (x = hi + lo to ~2^-48 relative)
 __global__ void k_split_x(const double* __restrict__ x, int64_t n_pad, float4* __restrict__ x2) {
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_pad; s += (int64_t)gridDim.x * blockDim.x) {
-    const double x0 = x[3 * s], x1 = x[3 * s + 1], x2c = x[3 * s + 2];
-    const float h0 = (float)x0, h1 = (float)x1, h2 = (float)x2c;
-    x2[2 * s] = make_float4(h0, h1, h2, 0.f);
-    x2[2 * s + 1] = make_float4((float)(x0 - (double)h0), (float)(x1 - (double)h1), (float)(x2c - (double)h2), 0.f);
+    const double v[3] = {x[3 * s], x[3 * s + 1], x[3 * s + 2]};
+    split_x(v, x2 + 2 * s);
   }
 }
 
@@ -387,8 +384,10 @@ sph_status ensure_operator(sph_neighbors* H, const sph_visc_params* P, cudaStrea
 }
 
 void launch_residual_f64(const sph_neighbors* H, int grid, const double* x, const double* b, double* r,
-                         double* partials, unsigned int* counter, double* res_out, cudaStream_t st) {
-  SPH_LAUNCH(k_split_x, grid_for(H, H->n_pad), kBlock, 0, st)(x, H->n_pad, H->v_x2.p);
+                         double* partials, unsigned int* counter, double* res_out, bool split, cudaStream_t st) {
+  if (split) {
+    SPH_LAUNCH(k_split_x, grid_for(H, H->n_pad), kBlock, 0, st)(x, H->n_pad, H->v_x2.p);
+  }
   if (H->op_tile_valid) {
     tile_residual(H, H->v_x2.p, x, b, r, partials, counter, res_out, st);
     return;

@@ -714,20 +714,6 @@ __global__ void __launch_bounds__(kBlock) k_cg_xr(int64_t n_pad, Vecs V, const f
   }
 }
 
-// identity rows (dynamic walls) take x = b before a CG solve: their exact value,
-// which keeps the wall rows of every residual zero, so the iteration only ever
-// sees the symmetric fluid block (the reduced system of Sec. 4)
-__global__ void k_identity_rows_take_b(const uint8_t* __restrict__ kind, int64_t n_pad, const double* __restrict__ b,
-                                       double* __restrict__ x) {
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_pad; s += (int64_t)gridDim.x * blockDim.x) {
-    if (kind[s] == KIND_IDENTITY) {
-      x[3 * s] = b[3 * s];
-      x[3 * s + 1] = b[3 * s + 1];
-      x[3 * s + 2] = b[3 * s + 2];
-    }
-  }
-}
-
 // x64 += d
 __global__ void k_add_correction(int64_t n_pad, const float4* __restrict__ d, double* __restrict__ x) {
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_pad; s += (int64_t)gridDim.x * blockDim.x) {
@@ -735,20 +721,6 @@ __global__ void k_add_correction(int64_t n_pad, const float4* __restrict__ d, do
     x[3 * s] += (double)v.x;
     x[3 * s + 1] += (double)v.y;
     x[3 * s + 2] += (double)v.z;
-  }
-}
-
-__global__ void k_gather_d3(const double* __restrict__ src, const int32_t* __restrict__ perm, int64_t n, int64_t n_pad,
-                            double* __restrict__ dst) {
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_pad; s += (int64_t)gridDim.x * blockDim.x) {
-    if (s < n) {
-      const int64_t i = perm[s];
-      dst[3 * s] = src[3 * i];
-      dst[3 * s + 1] = src[3 * i + 1];
-      dst[3 * s + 2] = src[3 * i + 2];
-    } else {
-      dst[3 * s] = dst[3 * s + 1] = dst[3 * s + 2] = 0.0;
-    }
   }
 }
 
@@ -762,14 +734,35 @@ __global__ void k_scatter_d3(const double* __restrict__ src, const int32_t* __re
   }
 }
 
-// squares per component of an [n_pad][3] float64 array, grid-reduced into out[3]
-__global__ void __launch_bounds__(kBlock) k_norm2_d3(const double* __restrict__ a, int64_t n_pad, double* partials,
+// What a solve starts from, in one pass over the rows: b and x from the caller's order
+// into the sorted one, x's float32 halves for the residual, and ||b||^2 per component
+// (out[3]).  Rows of kind `take_b` (dynamic walls before a CG solve, where kind is given)
+// take x = b: their exact value, which keeps the wall rows of every residual zero, so the
+// iteration only ever sees the symmetric fluid block (the reduced system of Sec. 4).
+__global__ void __launch_bounds__(kBlock) k_start_d3(const double* __restrict__ b, const double* __restrict__ x,
+                                                     const int32_t* __restrict__ perm, const uint8_t* __restrict__ kind,
+                                                     int64_t n, int64_t n_pad, double* __restrict__ b64,
+                                                     double* __restrict__ x64, float4* __restrict__ x2, double* partials,
                                                      unsigned int* counter, double* out) {
   double acc[3] = {0.0, 0.0, 0.0};
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_pad; s += (int64_t)gridDim.x * blockDim.x) {
-    acc[0] += a[3 * s] * a[3 * s];
-    acc[1] += a[3 * s + 1] * a[3 * s + 1];
-    acc[2] += a[3 * s + 2] * a[3 * s + 2];
+    double bv[3] = {0.0, 0.0, 0.0}, xv[3] = {0.0, 0.0, 0.0};
+    if (s < n) {
+      const int64_t i = perm[s];
+      const bool take_b = kind != nullptr && kind[s] == KIND_IDENTITY;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        bv[c] = b[3 * i + c];
+        xv[c] = take_b ? bv[c] : x[3 * i + c];
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      b64[3 * s + c] = bv[c];
+      x64[3 * s + c] = xv[c];
+      acc[c] += bv[c] * bv[c];
+    }
+    split_x(xv, x2 + 2 * s);
   }
   block_partials_f64<3>(acc, partials + (size_t)blockIdx.x * kMaxDots);
   if (arrive_last(counter)) {
@@ -838,15 +831,32 @@ static sph_status residual_update(sph_neighbors* H, cudaStream_t st, const float
   return SPH_OK;
 }
 
-// r64 = b64 - A x64 and rr[3] into H->host_flags area (synchronises)
-static sph_status true_residual(sph_neighbors* H, cudaStream_t st, double rr[3]) {
+// r64 = b64 - A x64 and its squares into rr[3] (synchronises); split: x64's float32
+// halves have to be made first
+static sph_status true_residual(sph_neighbors* H, cudaStream_t st, double rr[3], bool split = true, double* bb = nullptr) {
   const int grid = red_grid_for(H, H->n_pad);
   double* dev_out = reinterpret_cast<double*>(H->scal.p) + offsetof(SolverScalars, dots) / sizeof(double);
-  launch_residual_f64(H, grid, H->x64.p, H->b64.p, H->r64.p, H->partials.p, H->counters.p + CNT_RES, dev_out, st);
+  double* host = H->host_scal->dots;
+  launch_residual_f64(H, grid, H->x64.p, H->b64.p, H->r64.p, H->partials.p, H->counters.p + CNT_RES, dev_out, split, st);
   SPH_TRY_CUDA(cudaGetLastError());
-  SPH_TRY_CUDA(cudaMemcpyAsync(rr, dev_out, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
+  SPH_TRY_CUDA(cudaMemcpyAsync(host, dev_out, (bb ? 6 : 3) * sizeof(double), cudaMemcpyDeviceToHost, st));
   SPH_TRY_CUDA(cudaStreamSynchronize(st));
+  for (int c = 0; c < 3; ++c) rr[c] = host[c];
+  for (int c = 0; bb && c < 3; ++c) bb[c] = host[3 + c];
   return SPH_OK;
+}
+
+// b and x of a solve in sorted order, r64 = b - A x, and the squares of r64 and b: two
+// launches and one read-back (five launches and two before; 4% of a step of 1.4k rows)
+static sph_status start_residual(sph_neighbors* H, const double* b, const double* x, bool take_b, double rr[3],
+                                 double bb[3], cudaStream_t st) {
+  static_assert(kMaxDots >= 6, "dots hold both norms");
+  double* dev_bb = reinterpret_cast<double*>(H->scal.p) + offsetof(SolverScalars, dots) / sizeof(double) + 3;
+  SPH_LAUNCH(k_start_d3, red_grid_for(H, H->n_pad), kBlock, 0, st)(
+      b, x, H->perm.p, take_b ? H->op_kind.p : nullptr, H->n, H->n_pad, H->b64.p, H->x64.p, H->v_x2.p, H->partials.p,
+      H->counters.p + CNT_NORM, dev_bb);
+  SPH_TRY_CUDA(cudaGetLastError());
+  return true_residual(H, st, rr, false, bb);
 }
 
 // a kernel of the BiCGSTAB loop: a programmatic dependent launch unless the
@@ -981,16 +991,8 @@ sph_status solve_mixed(sph_neighbors* H, const sph_visc_params* P, const sph_sol
   unsigned int* C = H->counters.p;
   SPH_TRY_CUDA(cudaMemsetAsync(&S->fault, 0, sizeof(int32_t), st));
 
-  SPH_LAUNCH(k_gather_d3, grid_for(H, np), kBlock, 0, st)(b, H->perm.p, H->n, np, H->b64.p);
-  SPH_LAUNCH(k_gather_d3, grid_for(H, np), kBlock, 0, st)(x, H->perm.p, H->n, np, H->x64.p);
-  if (cg) SPH_LAUNCH(k_identity_rows_take_b, grid_for(H, np), kBlock, 0, st)(H->op_kind.p, np, H->b64.p, H->x64.p);
-  SPH_TRY_CUDA(cudaGetLastError());
-  double* dev_dots = reinterpret_cast<double*>(S) + offsetof(SolverScalars, dots) / sizeof(double);
-  SPH_LAUNCH(k_norm2_d3, grid_rows, kBlock, 0, st)(H->b64.p, np, H->partials.p, C + CNT_NORM, dev_dots);
-  SPH_TRY_CUDA(cudaGetLastError());
-  double bb[3];
-  SPH_TRY_CUDA(cudaMemcpyAsync(bb, dev_dots, sizeof(bb), cudaMemcpyDeviceToHost, st));
-  SPH_TRY_CUDA(cudaStreamSynchronize(st));
+  double bb[3], rr[3] = {0, 0, 0};
+  SPH_TRY(start_residual(H, b, x, cg, rr, bb, st));
   const double bnorm = std::sqrt(bb[0] + bb[1] + bb[2]);
 
   const double rtol = O->rtol > 0.0 ? O->rtol : 1e-6;
@@ -1027,12 +1029,11 @@ sph_status solve_mixed(sph_neighbors* H, const sph_visc_params* P, const sph_sol
     H->pass_slot_next = slot ^ 1;
   }
   const int* hist = H->pass_len[slot];
-  double rr[3] = {0, 0, 0};
   sph_status status = SPH_NOT_CONVERGED;
   // r64 after a pass comes from the update r64 -= A d (rr_full = false); the
   // first residual, the one that accepts the solution and the one reported are
   // recomputed as b - A x64 from x (rr_full = true)
-  bool rr_full = false, have_rr = false;
+  bool rr_full = true, have_rr = true;
   for (int ref = 0;; ++ref) {
     if (!have_rr) {
       SPH_TRY(true_residual(H, st, rr));
@@ -1186,11 +1187,8 @@ sph_status visc_residual(sph_neighbors* H, const sph_visc_params* P, const doubl
   SPH_TRY(ensure_operator(H, P, st));
   SPH_TRY(ensure_workspace(H));
   const int64_t np = H->n_pad;
-  SPH_LAUNCH(k_gather_d3, grid_for(H, np), kBlock, 0, st)(b, H->perm.p, H->n, np, H->b64.p);
-  SPH_LAUNCH(k_gather_d3, grid_for(H, np), kBlock, 0, st)(x, H->perm.p, H->n, np, H->x64.p);
-  SPH_TRY_CUDA(cudaGetLastError());
-  double rr[3];
-  SPH_TRY(true_residual(H, st, rr));
+  double rr[3], bb[3];
+  SPH_TRY(start_residual(H, b, x, false, rr, bb, st));
   SPH_LAUNCH(k_scatter_d3, grid_for(H, H->n), kBlock, 0, st)(H->r64.p, H->perm.p, H->n, r);
   SPH_TRY_CUDA(cudaGetLastError());
   return SPH_OK;

@@ -298,7 +298,7 @@ sph_status solve_fp64(sph_neighbors* H, const sph_visc_params* P, const sph_solv
   double rr[3] = {0, 0, 0};
   sph_status status = SPH_NOT_CONVERGED;
   for (int ref = 0;; ++ref) {
-    launch_residual_f64(H, grid_slices, H->x64.p, H->b64.p, H->r64.p, H->partials.p, C + C64_RES, dev_dots, st);
+    launch_residual_f64(H, grid_slices, H->x64.p, H->b64.p, H->r64.p, H->partials.p, C + C64_RES, dev_dots, true, st);
     SPH_TRY_CUDA(cudaGetLastError());
     SPH_TRY_CUDA(cudaMemcpyAsync(rr, dev_dots, sizeof(rr), cudaMemcpyDeviceToHost, st));
     SPH_TRY_CUDA(cudaStreamSynchronize(st));

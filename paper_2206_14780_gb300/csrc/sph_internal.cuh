@@ -339,8 +339,9 @@ sph_status build_neighbors(const sph_scene* sc, int32_t maxnb, sph_neighbors** o
 sph_status export_neighbors(const sph_neighbors* H, int64_t* offsets, int32_t* idx, cudaStream_t st);
 
 // operator.cu
+// split: make x's float32 halves (v_x2) first
 void launch_residual_f64(const sph_neighbors* H, int grid, const double* x, const double* b, double* r,
-                         double* partials, unsigned int* counter, double* res_out, cudaStream_t st);
+                         double* partials, unsigned int* counter, double* res_out, bool split, cudaStream_t st);
 // r -= A d (sorted [n_pad][3] float64 r, float32 d), same reduction outputs
 void launch_residual_update(const sph_neighbors* H, int grid, const float4* d, double* r, double* partials,
                             unsigned int* counter, double* res_out, cudaStream_t st);
