@@ -167,37 +167,44 @@ __device__ __forceinline__ void tile_rows(const BatchView& B, int t, int64_t& fi
 
 // ---- the tile form inside a batch tile -----------------------------------------------
 // A batch tile of a scene is a run of that scene's tiles (16, 32 and 64 slices are
-// whole numbers of 1, 2, 4 or 8): the block takes them one after the other, each with its
-// union in shared memory and 8 / ts threads per row.
+// whole numbers of 1, 2, 4 or 8): the block takes them one after the other, one-slice
+// tiles two at a time, each with its union in shared memory and 8 / step threads per row
+// (one at a time, a batch of 4 scenes with one of 4k rows took 9% longer).
+__device__ __forceinline__ int tile_step(const SceneDesc& d) { return d.ts > 1 ? d.ts : 2; }
 struct TileLane {
-  int split, splits, row, rows;   // the thread's share of a row and its row in the tile
-  int64_t sl, s;                  // slice and row in the scene
+  int split, splits, row, rows;   // the thread's share of a row and its row in the step
+  int n0, n1, ubase;              // union sizes of the step's tiles, where the row's union starts
+  int64_t tile, sl, s;            // first tile, slice and row in the scene
   bool have;
 };
-__device__ __forceinline__ TileLane tile_lane(const SceneDesc& d, int64_t tile) {
+__device__ __forceinline__ TileLane tile_lane(const SceneDesc& d, int64_t slice0) {
   TileLane L;
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  L.splits = 8 / d.ts;
-  L.split = wid / d.ts;
-  L.row = (wid % d.ts) * 32 + lane;
-  L.rows = 32 * d.ts;
-  L.sl = tile * d.ts + wid % d.ts;
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, g = tile_step(d);
+  L.splits = 8 / g;
+  L.split = wid / g;
+  L.row = (wid % g) * 32 + lane;
+  L.rows = 32 * g;
+  L.tile = slice0 / d.ts;
+  L.n0 = d.tv.unum[L.tile];
+  L.n1 = d.ts == 1 && L.tile + 1 < d.tv.ntiles ? d.tv.unum[L.tile + 1] : 0;
+  L.sl = slice0 + wid % g;
+  L.ubase = d.ts == 1 && wid % g == 1 ? L.n0 : 0;
   L.s = L.sl * kSlice + lane;
   L.have = L.sl < d.tv.nslices;
   return L;
 }
 
 // fin(row, v_b, y) for the rows of batch tile [sl0, sl0 + nsl) of y = D^-1 A v; u: the
-// union, part: [7][32][3] floats, the most any ts takes
+// unions, part: [3][64][3] floats
 template <class Fin>
 __device__ __forceinline__ void batch_apply(const SceneDesc& d, const float4* __restrict__ v, int64_t sl0, int nsl,
                                             float4* u, float* part, Fin fin) {
   const TileView& op = d.tv;
   const int lane = threadIdx.x & 31;
-  for (int sub = 0; sub < nsl; sub += d.ts) {
-    const int64_t tile = (sl0 + sub) / d.ts;
-    tile_load_union(op, tile, v, u);
-    const TileLane L = tile_lane(d, tile);
+  for (int sub = 0; sub < nsl; sub += tile_step(d)) {
+    const TileLane L = tile_lane(d, sl0 + sub);
+    tile_load_union(op, L.tile, v, u);
+    if (L.n1 > 0) tile_load_union(op, L.tile + 1, v, u + L.n0);
     int c = 0;
     uint8_t kd = KIND_IDENTITY;
     float4 vb = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -212,7 +219,7 @@ __device__ __forceinline__ void batch_apply(const SceneDesc& d, const float4* __
     cp_async_wait_all();
     __syncthreads();
     float ax = 0.f, ay = 0.f, az = 0.f;
-    ts.sum(u, L.split, L.splits, kap * vb.x, kap * vb.y, kap * vb.z, ax, ay, az);
+    ts.sum(u + L.ubase, L.split, L.splits, kap * vb.x, kap * vb.y, kap * vb.z, ax, ay, az);
     if (L.splits > 1) {
       if (L.split > 0) {
         float* q = part + ((L.split - 1) * L.rows + L.row) * 3;
@@ -249,7 +256,7 @@ __global__ void __launch_bounds__(kBlock) kb_split(BatchView B, int64_t nrows) {
 template <bool TILE>
 __global__ void __launch_bounds__(kBlock) kb_residual(BatchView B) {
   extern __shared__ __align__(16) float4 dyn[];
-  __shared__ double rpart[TILE ? 224 * 3 : 1];
+  __shared__ double rpart[TILE ? 192 * 3 : 1];
   if (threadIdx.x == 0 && blockIdx.x == 0) {   // counted by kb_init
     B.ctrl->active = 0;
     B.ctrl->passes += 1;
@@ -276,17 +283,16 @@ __global__ void __launch_bounds__(kBlock) kb_residual(BatchView B) {
     };
     const float4* x2 = B.V.x2 + 2 * d.row_off;
     if (TILE) {
-      for (int sub = 0; sub < B.tile_nsl[t]; sub += d.ts) {
-        const int64_t tile = (B.tile_slice0[t] + sub) / d.ts;
-        const int nu = d.tv.unum[tile];
-        const int32_t* __restrict__ ids = d.tv.uni + tile * d.tv.ustride;
+      for (int sub = 0; sub < B.tile_nsl[t]; sub += tile_step(d)) {
+        const TileLane L = tile_lane(d, B.tile_slice0[t] + sub);
+        const int nu = L.n0 + L.n1;
+        const int32_t* __restrict__ ids = d.tv.uni + L.tile * d.tv.ustride;
         float4 *uh = dyn, *ul = dyn + nu;
         for (int i = threadIdx.x; i < nu; i += kBlock) {
-          const int64_t q = ids[i];
+          const int64_t q = i < L.n0 ? ids[i] : ids[d.tv.ustride + i - L.n0];
           cp_async16(uh + i, x2 + 2 * q);
           cp_async16(ul + i, x2 + 2 * q + 1);
         }
-        const TileLane L = tile_lane(d, tile);
         int c = 0;
         uint8_t k = KIND_IDENTITY;
         float4 bh = make_float4(0.f, 0.f, 0.f, 0.f), bl = bh;
@@ -301,7 +307,7 @@ __global__ void __launch_bounds__(kBlock) kb_residual(BatchView B) {
         __syncthreads();
         DFAcc a0, a1, a2;
         if (c > 0)
-          tile_residual_row<true>(d.tv, uh, ul, L.sl, lane, c, L.split, L.splits,
+          tile_residual_row<true>(d.tv, uh + L.ubase, ul + L.ubase, L.sl, lane, c, L.split, L.splits,
                                   make_float4(kap * bh.x, kap * bh.y, kap * bh.z, 0.f),
                                   make_float4(kap * bl.x, kap * bl.y, kap * bl.z, 0.f), a0, a1, a2);
         double v0 = a0.value(), v1 = a1.value(), v2 = a2.value();
@@ -404,7 +410,7 @@ __global__ void __launch_bounds__(kBlock) kb_init(BatchView B) {
 template <int U, bool PF, int NB, bool TILE>
 __global__ void __launch_bounds__(NB, TILE ? 4 : 1) kb_pass(BatchView B, int iter_cap) {
   extern __shared__ __align__(16) float4 dyn[];
-  __shared__ float part[TILE ? 224 * 3 : 1];
+  __shared__ float part[TILE ? 192 * 3 : 1];
   for (int it = 0; it < iter_cap; ++it) {
     if (*(volatile int32_t*)&B.ctrl->active == 0) break;
     // phase 1: p = r + beta p - alpha' Ap
@@ -806,7 +812,10 @@ sph_status sph_batch_create(sph_neighbors* const* handles, const sph_visc_params
   Bt->hdesc.assign(nscenes, SceneDesc{});
   int64_t rows = 0, max_tiles = 0;
   Bt->tile_form = true;
-  for (int s = 0; s < nscenes; ++s) Bt->tile_form = Bt->tile_form && handles[s] && handles[s]->tile_ok;
+  for (int s = 0; s < nscenes; ++s) {   // (two unions of one-slice tiles have to fit where one does)
+    const sph_neighbors* H = handles[s];
+    Bt->tile_form = Bt->tile_form && H && H->tile_ok && (H->tile_ts > 1 || 2 * H->tile_umax <= kTileUnion);
+  }
   for (int s = 0; s < nscenes; ++s) {
     sph_neighbors* H = handles[s];
     if (!H) {
@@ -827,8 +836,9 @@ sph_status sph_batch_create(sph_neighbors* const* handles, const sph_visc_params
     if (Bt->tile_form) {
       d.tv = tile_view(H);
       d.ts = H->tile_ts;
-      Bt->smem = std::max(Bt->smem, tile_smem(H, 16));
-      Bt->smem_res = std::max(Bt->smem_res, tile_smem(H, 32));
+      const int unions = d.ts > 1 ? 1 : 2;   // tile_step
+      Bt->smem = std::max(Bt->smem, tile_smem(H, 16) * unions);
+      Bt->smem_res = std::max(Bt->smem_res, tile_smem(H, 32) * unions);
     }
     if (H->row_scaled) {  // the preconditioner's diagonal D / s
       d.op.invD = d.tv.invD = H->invD_sc.p;
