@@ -157,3 +157,55 @@ def test_cooperative_solve_limits_and_stalls():
     x = torch.zeros_like(b)
     rep = nb.solve(params_for(s), binding.solve_opts(), zero, x)
     assert rep["status"] == 0 and rep["iters"] == 0 and float(x.abs().max()) == 0.0
+
+
+@pytest.mark.parametrize("make,maxnb", [
+    # either side of the one-slice rule: 151 and 152 slices (fewer tiles than SMs, or not)
+    (lambda: scenes.random_box(11, nf=151 * 32 - 5, nw_layers=0, mu_spread=3.0), 128),
+    (lambda: scenes.random_box(12, nf=152 * 32 - 5, nw_layers=0, mu_spread=3.0), 128),
+    # two slices per tile with walls, and with rows of ~250
+    (lambda: scenes.couette(13, nx=20, ny=16, nz=19), 128),
+    (lambda: scenes.couette(14, nx=18, ny=23, nz=18, layers=4, kernel=1), 320)])
+def test_one_and_two_slice_tiles(make, maxnb):
+    """Lists, apply, residual and a solve where the rule turns from one slice per tile to
+    two; tolerances as above, the solve's true residual by the oracle's matrix."""
+    torch = torch_cuda()
+    from paper_2206_14780_gb300 import binding
+
+    s = make()
+    nb, _ = lib_build(s, maxnb)
+    off, idx, A = oracle_system(s)
+    o, i = nb.export()
+    np.testing.assert_array_equal(o.cpu().numpy(), off)
+    np.testing.assert_array_equal(i.cpu().numpy(), idx)
+    v = np.zeros((s.n, 4), np.float32)
+    v[:, :3] = np.random.default_rng(15).normal(size=(s.n, 3))
+    yt = torch.empty((s.n, 4), device="cuda")
+    nb.apply(params_for(s), torch.from_numpy(v).cuda(), yt)
+    assert rel_l2(yt.cpu().numpy()[:, :3], A @ v[:, :3].astype(np.float64)) < 1e-5
+    x = torch.from_numpy(s.x0).cuda()
+    rep = nb.solve(params_for(s), binding.solve_opts(rtol=1e-8), torch.from_numpy(s.b).cuda(), x)
+    assert rep["status"] == 0, rep
+    assert oop.true_residual(A, x.cpu().numpy(), s.b)[0] <= 1.1e-8
+
+
+def test_region_sizes_follow_each_other_on_one_handle():
+    """A handle rebuilt on sets that need the small, the largest and again the small search
+    region (it starts with the size of its last rebuild), and the global scan in between."""
+    first = scenes.couette(2, nx=21, ny=9, nz=11)
+    nb, _ = lib_build(first)
+    for make, maxnb in (CASES["large_region"], (lambda: first, 128), CASES["sparse"], (lambda: first, 128), CASES["gaussian"]):
+        s = make()
+        t = _tensors(s)
+        nb.rebuild(t["pos"], t["rho"], t["mu"], t["ptype"], s.lo, s.hi, s.periodic, s.h, maxnb,
+                   kernel=getattr(s, "kernel", 0))
+        off, idx, _ = oracle_system(s)
+        o, i = nb.export()
+        np.testing.assert_array_equal(o.cpu().numpy(), off)
+        np.testing.assert_array_equal(i.cpu().numpy(), idx)
+
+
+def _tensors(s):
+    from paper_2206_14780_gb300 import binding
+
+    return binding.scene_tensors(s)
