@@ -193,7 +193,7 @@ def read_peaks():
 
 
 # the sources of the operator apply kernel (k_apply_dot and what it includes)
-TRAFFIC_SOURCES = ("apply.cuh", "solver.cu", "reduce.cuh", "bicgstab_scalars.cuh", "sph_internal.cuh")
+TRAFFIC_SOURCES = ("tiles.cuh", "solver.cu", "reduce.cuh", "bicgstab_scalars.cuh", "sph_internal.cuh")
 
 
 def apply_traffic(alg_bytes):
@@ -469,7 +469,8 @@ def run_sphvisc(args):
     traffic, traffic_src = apply_traffic(prof["apply_bytes"])
     roofline = dict(bound="hbm", achieved=achieved, peak=hbm, unit="GB/s",
                     frac=(achieved / hbm) if achieved else None, traffic=traffic, traffic_source=traffic_src,
-                    kernel="k_apply_dot (operator apply + fused dots)", peak_source=peak_kind,
+                    kernel="k_tile_apply_dot (operator apply + fused dots)" if prof["apply_variant"][0] == 6
+                    else "k_apply_dot (operator apply + fused dots)", peak_source=peak_kind,
                     apply_launches=prof["apply_launches"], apply_avg_us=avg_apply_ms * 1e3,
                     apply_avg_us_Ap=1e3 * prof["phase_ms"][0] / max(1, prof["phase_launches"][0]),
                     apply_avg_us_Ars=1e3 * prof["phase_ms"][1] / max(1, prof["phase_launches"][1]),
@@ -1101,7 +1102,7 @@ def run_apply_forms(nb, params, n, dev, reps=20):
         us = 1e3 * c["standalone_ms"][k] / max(1, c["standalone_launches"][k])
         out[name] = dict(us_per_apply=us, algorithmic_bytes=int(nbytes), gbs=nbytes / (us * 1e-6) / 1e9,
                          launches=c["standalone_launches"][k])
-    out["note"] = ("y = A v alone (no fused dots); stored: 8 B per coefficient + 41 B per row; on the fly: "
+    out["note"] = ("y = A v alone (no fused dots); stored: 6 B per coefficient (8 where the lists have no tile form) + 41 B per row; on the fly: "
                    "4 B per neighbour-list entry + 61 B per row, coefficients recomputed in float32")
     return out
 

@@ -703,10 +703,11 @@ typedef struct {
   int64_t launches;        /* kernels this library launched (all handles, all calls) */
   int64_t apply_launches;  /* operator applies timed on this handle (the sample)     */
   double apply_ms;         /* summed device time of those applies (ms)               */
-  int64_t apply_bytes;     /* algorithmic bytes of one apply: 8 per stored
-                              coefficient (index + value) plus, per row, 16 read of
-                              v, 16 write of the result, 16 read of r0^ for the dot
-                              and 9 of row data (count, kind, 1/D)                  */
+  int64_t apply_bytes;     /* algorithmic bytes of one apply: 6 per stored
+                              coefficient in the tile form (16-bit position and
+                              value), 8 in the others (index and value), plus, per
+                              row, 16 read of v, 16 write of the result, 16 read of
+                              r0^ for the dot and 9 of row data (count, kind, 1/D)  */
   int64_t op_nnz;          /* stored coefficients of A(dt)                          */
   int64_t phase_launches[2]; /* apply_launches split: [0] A p (delta), [1] A r* (omega) */
   double phase_ms[2];        /* apply_ms split the same way                           */

@@ -379,7 +379,8 @@ sph_status sph_profile_read(sph_neighbors* h, sph_profile_counters* out, int32_t
       h->op_nnz = (int64_t)c;
     }
     out->op_nnz = h->op_nnz;
-    out->apply_bytes = 8 * h->op_nnz + (16 + 16 + 16 + 9) * h->n;
+    const bool tiles = h->tile_grid > 0 || (h->op_tile_valid && !h->op_ih_valid);
+    out->apply_bytes = (tiles ? 6 : 8) * h->op_nnz + (16 + 16 + 16 + 9) * h->n;
     for (int k = 0; k < 2; ++k) {
       out->phase_launches[k] = h->prof_n_ph[k];
       out->phase_ms[k] = h->prof_ms_ph[k];
