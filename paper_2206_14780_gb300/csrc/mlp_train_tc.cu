@@ -27,6 +27,8 @@
 //     epilogue overwrites their operand), and the last one of a tile is issued with
 //     the next tile's first product.  That tile's features are copied (cp.async) into
 //     the buffer of this tile's output deltas meanwhile; the two swap roles per tile.
+// 262k rows: 49.5 -> 27.0 million warp instructions, 103 -> 74 us against eight hand-overs
+// at which every thread waited for every MMA, with one row per thread.
 //
 // Tensor memory (256 columns per CTA): Z (64) holds the forward's pre-activations in
 // turn and, in the backward pass, Z_2 and Z_1 (recomputed by the same MMAs, so SiLU'

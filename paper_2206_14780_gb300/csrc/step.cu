@@ -96,7 +96,8 @@ __device__ __forceinline__ float kernel_w(float q, const StepGeom& g) {
 // number from 2 to 16 (7 for water), else 0.  A float64 instruction costs a warp ~63
 // cycles and pow over a hundred of them; x^k by squaring is 4 at k = 7, and the root one
 // Halley step from the float32 root (error (k^2 - 1) / 12 e^3 of its ~3e-7), both within
-// a few units of float64's last place before the result is rounded to float32.
+// a few units of float64's last place before the result is rounded to float32.  The
+// pressures of 91k rows took 26 us with pow, the walls' 37 us are 29 us with the root.
 struct Zeta {
   double z;
   int k;
