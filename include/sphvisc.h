@@ -118,7 +118,9 @@ typedef struct sph_neighbors sph_neighbors;
  *   entry points that walk 32-bit rows (export, the on-the-fly apply, features),
  *   take 4 * max_neighbors bytes more.
  * Copies pos/rho/mu/ptype into the handle: the scene arrays may be freed after
- * the call returns. */
+ * the call returns.  A rebuild that fails once it has begun (SPH_ERR_CAPACITY,
+ * SPH_ERR_NONFINITE, a CUDA error) leaves the handle without lists: calls that need
+ * them return SPH_ERR_INVALID until a build on it succeeds. */
 sph_status sph_build_neighbors(const sph_scene* scene, int32_t max_neighbors,
                                sph_neighbors** handle, void* stream);
 

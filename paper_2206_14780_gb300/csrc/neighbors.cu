@@ -1012,7 +1012,14 @@ static sph_status fixed_offsets(sph_neighbors* H, cudaStream_t st) {
   return SPH_OK;
 }
 
+sph_status require_lists(const sph_neighbors* H) {
+  if (H->lists_ok) return SPH_OK;
+  set_error("the last sph_build_neighbors on this handle failed: it has no neighbour lists until a build succeeds");
+  return SPH_ERR_INVALID;
+}
+
 sph_status ensure_nbr(sph_neighbors* H, cudaStream_t st) {
+  SPH_TRY(require_lists(H));
   if (H->nbr_valid) return SPH_OK;
   SPH_TRY(H->nbr.alloc(H->n_pad * (int64_t)H->maxnb));
   SPH_TRY(fixed_offsets(H, st));
@@ -1149,6 +1156,7 @@ sph_status build_neighbors(const sph_scene* sc, int32_t maxnb, sph_neighbors** o
   TRYF_CUDA(cudaGetDevice(&H->device));
   TRYF_CUDA(cudaDeviceGetAttribute(&H->num_sms, cudaDevAttrMultiProcessorCount, H->device));
   const int64_t n = sc->n;
+  H->lists_ok = false;
   if (H->row_scaled && H->n != n) {   // a caller-order row scale no longer fits
     H->row_scaled = false;
     ++H->rs_version;
@@ -1281,6 +1289,7 @@ sph_status build_neighbors(const sph_scene* sc, int32_t maxnb, sph_neighbors** o
   H->nnz = total;
   H->nnz_pad = total_pad;
   H->max_cnt = maxc;
+  H->lists_ok = true;
   *out = H;
   return SPH_OK;
 #undef TRYF
@@ -1292,6 +1301,7 @@ sph_status export_neighbors(const sph_neighbors* H, int64_t* offsets, int32_t* i
     set_error("sph_neighbors_export: null argument");
     return SPH_ERR_INVALID;
   }
+  SPH_TRY(require_lists(H));
   sph_neighbors* M = const_cast<sph_neighbors*>(H);
   SPH_TRY(M->tmp_i32a.alloc(H->n));
   int grid = grid_for(H, H->n);

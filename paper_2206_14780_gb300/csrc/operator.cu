@@ -358,6 +358,7 @@ sph_status ensure_operator(sph_neighbors* H, const sph_visc_params* P, cudaStrea
     set_error("viscous parameters: dt must be positive and finite, boundary/mean one of the enums");
     return SPH_ERR_INVALID;
   }
+  SPH_TRY(require_lists(H));
   const bool tile = form == OP_FAST && H->tile_ok;
   const bool same = H->op_valid && H->op_params.dt == P->dt && H->op_params.boundary == P->boundary &&
                     H->op_params.mean == P->mean && H->op_mu_version == H->mu_version;

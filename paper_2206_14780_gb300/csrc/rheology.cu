@@ -188,6 +188,7 @@ __global__ void __launch_bounds__(256) k_tile_mu(TileView op, const int32_t* __r
 }  // namespace
 
 sph_status set_viscosity_impl(sph_neighbors* H, const float* mu, cudaStream_t st) {
+  SPH_TRY(require_lists(H));
   SPH_TRY_CUDA(cudaMemsetAsync(H->flags.p, 0, sizeof(int32_t), st));
   SPH_LAUNCH(k_set_mu, grid_for(H, H->n), kBlock, 0, st)(mu, H->perm.p, H->n, H->mu_s.p, H->flags.p);
   SPH_TRY_CUDA(cudaGetLastError());
@@ -204,6 +205,7 @@ sph_status set_viscosity_impl(sph_neighbors* H, const float* mu, cudaStream_t st
 
 sph_status mu_papanastasiou(sph_neighbors* H, const float* vel, const float* wall_vel, double tau0, double mu0,
                             double m, float* mu_out, int set_handle, cudaStream_t st) {
+  SPH_TRY(require_lists(H));
   if (!H->tile_ok) SPH_TRY(ensure_nbr(H, st));
   MuGeom g{};
   for (int ax = 0; ax < 3; ++ax) {

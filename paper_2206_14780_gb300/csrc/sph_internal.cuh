@@ -197,6 +197,10 @@ struct sph_neighbors {
   int64_t nnz = 0, nnz_pad = 0;
   int32_t max_cnt = 0;
 
+  // false from the start of a (re)build to its success: a build that fails leaves lists
+  // and sorted copies that do not belong together, and no entry point reads them
+  bool lists_ok = false;
+
   // The lists above are kept as 16-bit positions per tile (tiles.cuh) where the
   // particle set allows it (tile_ok); nbr and slice_off are then made on demand
   // (ensure_nbr) for the kernels that walk 32-bit rows.
@@ -330,6 +334,8 @@ struct sph_neighbors {
 namespace sph {
 
 // neighbors.cu
+// SPH_ERR_INVALID while the handle's last build has not succeeded
+sph_status require_lists(const sph_neighbors* H);
 // the 32-bit rows of the lists (nbr, slice_off), expanded from the tiles if need be
 sph_status ensure_nbr(sph_neighbors* H, cudaStream_t st);
 
