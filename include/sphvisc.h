@@ -437,8 +437,9 @@ sph_status sph_step(sph_state* state, const sph_step_params* params, const sph_s
 typedef struct sph_batch sph_batch;
 
 /* handles: (host) [nscenes] built handles; params: (host) [nscenes] A(dt)
- * parameters (set up on each handle here; a handle rebuilt or given new
- * viscosities afterwards makes sph_batch_solve fail with SPH_ERR_INVALID).
+ * parameters (set up on each handle here; a handle that was rebuilt, given new
+ * viscosities or is set up for other parameters makes sph_batch_solve fail with
+ * SPH_ERR_INVALID).
  * The batch keeps pointers to the handles: destroy it before them. */
 sph_status sph_batch_create(sph_neighbors* const* handles, const sph_visc_params* params,
                             int32_t nscenes, sph_batch** batch, void* stream);

@@ -654,6 +654,7 @@ struct sph_batch {
   std::vector<sph_visc_params> params;
   std::vector<int64_t> row_off;
   std::vector<uint64_t> rs_version;   // each handle's row-scale version at creation
+  std::vector<uint64_t> list_version; // and its build count: the tiles, ts and smem below are those lists'
   bool tile_form = false;             // every scene's operator is in the tile form
   size_t smem = 0, smem_res = 0;      // dynamic shared memory of the pass and the residual kernels
   DBuf<double> norms;                 // [nscenes][kNormBlocks][3]
@@ -754,6 +755,31 @@ sph_status enqueue_pass(sph_batch* Bt, const BatchView& B, int cap, cudaStream_t
 // shorter), uploads the tile table and the descriptors' tile ranges, and sizes
 // each variant's co-resident grid.  The device arrays hold the tiles of the
 // shortest candidate.
+// A scene's operator arrays as they are now: a set-up at other parameters and back may
+// have moved them, so every solve takes them afresh.
+void scene_view(const sph_batch* Bt, const sph_neighbors* H, SceneDesc& d) {
+  d.op = op_view(H);
+  d.op_lo = H->op_lo.p;
+  d.D64 = H->D64.p;
+  if (Bt->tile_form) d.tv = tile_view(H);
+  if (H->row_scaled) {  // the preconditioner's diagonal D / s
+    d.op.invD = d.tv.invD = H->invD_sc.p;
+    d.D64 = H->D64_sc.p;
+  }
+}
+
+// Whether a scene's handle still is what the batch was made for: the same lists (the
+// kernels' shared memory and tile sizes are theirs), A(dt) of the scene's parameters in
+// the batch's form, the same row scale.
+bool scene_unchanged(const sph_batch* Bt, int s) {
+  const sph_neighbors* H = Bt->handles[s];
+  const sph_visc_params& P = Bt->params[s];
+  return H->lists_ok && H->list_version == Bt->list_version[s] && H->op_valid &&
+         (Bt->tile_form ? H->op_tile_valid : H->op_ih_valid) && H->op_mu_version == H->mu_version &&
+         H->op_params.dt == P.dt && H->op_params.boundary == P.boundary && H->op_params.mean == P.mean &&
+         H->rs_version == Bt->rs_version[s] && (!H->row_scaled || H->rs_op_version == H->op_version);
+}
+
 sph_status build_tiles(sph_batch* Bt, int ti, cudaStream_t st) {
   const int64_t T = kTileCands[ti];
   std::vector<int32_t> ts, t0, tn;
@@ -829,20 +855,14 @@ sph_status sph_batch_create(sph_neighbors* const* handles, const sph_visc_params
     Bt->params.push_back(params[s]);
     Bt->row_off.push_back(rows);
     Bt->rs_version.push_back(H->rs_version);
+    Bt->list_version.push_back(H->list_version);
     SceneDesc& d = Bt->hdesc[s];
-    d.op = op_view(H);
-    d.op_lo = H->op_lo.p;
-    d.D64 = H->D64.p;
+    scene_view(Bt, H, d);
     if (Bt->tile_form) {
-      d.tv = tile_view(H);
       d.ts = H->tile_ts;
       const int unions = d.ts > 1 ? 1 : 2;   // tile_step
       Bt->smem = std::max(Bt->smem, tile_smem(H, 16) * unions);
       Bt->smem_res = std::max(Bt->smem_res, tile_smem(H, 32) * unions);
-    }
-    if (H->row_scaled) {  // the preconditioner's diagonal D / s
-      d.op.invD = d.tv.invD = H->invD_sc.p;
-      d.D64 = H->D64_sc.p;
     }
     d.row_off = rows;
     d.n = H->n;
@@ -953,13 +973,14 @@ sph_status sph_batch_solve(sph_batch* Bt, const sph_solve_opts* O, const double*
       set_error("sph_batch_solve: b/x of scene %d is null", s);
       return SPH_ERR_INVALID;
     }
-    sph_neighbors* H = Bt->handles[s];
-    // the operator may have been rebuilt since the batch was made
-    if (!H->op_valid || !(Bt->tile_form ? H->op_tile_valid : H->op_ih_valid) || H->op_mu_version != H->mu_version || H->rs_version != Bt->rs_version[s] ||
-        (H->row_scaled && H->rs_op_version != H->op_version)) {
+    if (!scene_unchanged(Bt, s)) {
       set_error("sph_batch_solve: scene %d's handle changed after sph_batch_create", s);
       return SPH_ERR_INVALID;
     }
+  }
+  for (int s = 0; s < S; ++s) {
+    const sph_neighbors* H = Bt->handles[s];
+    scene_view(Bt, H, Bt->hdesc[s]);
     const int64_t o = Bt->row_off[s];
     SPH_LAUNCH(kb_gather, grid_for(H, H->n_pad), kBlock, 0, st)(b[s], H->perm.p, H->n, H->n_pad,
                                                                   Bt->dvec.p + 3 * N + 3 * o);

@@ -1157,6 +1157,7 @@ sph_status build_neighbors(const sph_scene* sc, int32_t maxnb, sph_neighbors** o
   TRYF_CUDA(cudaDeviceGetAttribute(&H->num_sms, cudaDevAttrMultiProcessorCount, H->device));
   const int64_t n = sc->n;
   H->lists_ok = false;
+  ++H->list_version;
   if (H->row_scaled && H->n != n) {   // a caller-order row scale no longer fits
     H->row_scaled = false;
     ++H->rs_version;

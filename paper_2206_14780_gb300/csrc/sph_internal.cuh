@@ -200,6 +200,7 @@ struct sph_neighbors {
   // false from the start of a (re)build to its success: a build that fails leaves lists
   // and sorted copies that do not belong together, and no entry point reads them
   bool lists_ok = false;
+  uint64_t list_version = 0;       // counts the (re)builds
 
   // The lists above are kept as 16-bit positions per tile (tiles.cuh) where the
   // particle set allows it (tile_ok); nbr and slice_off are then made on demand
