@@ -825,17 +825,36 @@ __global__ void __launch_bounds__(256) k_tile_plan(const uint8_t* __restrict__ t
   nfl[s] = nf;
 }
 
-// the lists as 32-bit rows in the fixed-capacity SELL-32 layout of k_neighbors
-__global__ void k_tile_expand(const uint16_t* __restrict__ idx, int64_t istride, const int32_t* __restrict__ cnt,
-                              const int32_t* __restrict__ nfl, const int32_t* __restrict__ uni, int32_t ustride,
-                              int rows_per_tile, int64_t n, int32_t maxnb, int32_t* __restrict__ nbr) {
-  for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
-    const int lane = (int)(s % kSlice), c = cnt[s], nf = nfl[s], gap = ((nf + 3) & ~3) - nf;
-    const uint16_t* __restrict__ mine = idx + (s / kSlice) * istride;
-    const int32_t* __restrict__ u = uni + (s / rows_per_tile) * ustride;
-    const int64_t base = (s / kSlice) * (int64_t)kSlice * maxnb + lane;
-    for (int j = 0; j < c; ++j)
-      nbr[base + (int64_t)j * kSlice] = u[mine[tile_entry(j < nf ? j : j + gap, lane)] >> 4];
+// The lists as 32-bit rows in the fixed-capacity SELL-32 layout of k_neighbors and in its
+// order, from the search's region places (raw has that layout and order), so that what
+// sums along them does not depend on how the lists were made.  The plan's entries are
+// ordered for shared-memory banks; rows expanded from those cost the export's sort most
+// (rebuild and export of 77k rows of ~250: 7.69 ms against 6.50, 12k: 3.43 against 2.97)
+// and the on-the-fly apply a little (rebuild and apply, 58k rows: 352 against 332 us),
+// while set-ups along 32-bit rows are 3-6% faster on them (rebuild and row norms, 58k:
+// 435 against 452 us).  One block per tile: the region's rows into shared memory, then
+// one coalesced pass over the entries.
+__global__ void __launch_bounds__(256) k_tile_expand(const uint16_t* __restrict__ raw, const int2* __restrict__ tcells,
+                                                     const int32_t* __restrict__ tncell, const int32_t* __restrict__ cnt,
+                                                     int slices_per_tile, int64_t nslices, int64_t n, int32_t maxnb,
+                                                     int32_t* __restrict__ nbr) {
+  extern __shared__ int32_t place[];   // region place -> row
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t tile = blockIdx.x;
+  const int2* __restrict__ cells = tcells + tile * (kTileCells + 1);
+  const int m = tncell[tile];
+  for (int q = wid; q < m; q += 8) {
+    const int2 a = cells[q];
+    for (int k = lane; k < a.y >> 16; k += 32) place[(a.y & 0xffff) + k] = a.x + k;
+  }
+  __syncthreads();
+  const int64_t sl1 = min((tile + 1) * slices_per_tile, nslices);
+  for (int64_t sl = tile * slices_per_tile; sl < sl1; ++sl) {
+    const int64_t s = sl * kSlice + lane, base = sl * kSlice * (int64_t)maxnb + lane;
+    const int c = s < n ? cnt[s] : 0, most = __reduce_max_sync(0xffffffffu, c);
+#pragma unroll 4
+    for (int j = wid; j < most; j += 8)
+      if (j < c) nbr[base + (int64_t)j * kSlice] = place[raw[base + (int64_t)j * kSlice]];
   }
 }
 
@@ -1023,8 +1042,8 @@ sph_status ensure_nbr(sph_neighbors* H, cudaStream_t st) {
   if (H->nbr_valid) return SPH_OK;
   SPH_TRY(H->nbr.alloc(H->n_pad * (int64_t)H->maxnb));
   SPH_TRY(fixed_offsets(H, st));
-  SPH_LAUNCH(k_tile_expand, grid_for(H, H->n), kBlock, 0, st)(H->t_idx.p, H->t_istride, H->cnt.p, H->t_nfl.p, H->t_uni.p,
-                                                              H->t_ustride, 32 * H->tile_ts, H->n, H->maxnb, H->nbr.p);
+  SPH_LAUNCH(k_tile_expand, (int)H->ntiles, 256, H->tile_cap * sizeof(int32_t), st)(
+      H->t_raw.p, H->t_cells.p, H->t_ncell.p, H->cnt.p, H->tile_ts, H->nslices, H->n, H->maxnb, H->nbr.p);
   SPH_TRY_CUDA(cudaGetLastError());
   H->nbr_valid = true;
   return SPH_OK;
@@ -1058,6 +1077,7 @@ static sph_status launch_tile_search(sph_neighbors* H, const Grid& g, const Band
                                      cudaStream_t st) {
   const int ts = tile_slices_for(H->nslices, maxnb, H->num_sms);
   H->tile_ts = ts;
+  H->tile_cap = cap;
   H->ntiles = (H->nslices + ts - 1) / ts;
   H->t_istride = 32 * (((maxnb + 3) & ~3) + 4);
   H->t_ustride = cap < kTileUnion + 1 ? cap : kTileUnion + 1;

@@ -204,15 +204,16 @@ struct sph_neighbors {
 
   // The lists above are kept as 16-bit positions per tile (tiles.cuh) where the
   // particle set allows it (tile_ok); nbr and slice_off are then made on demand
-  // (ensure_nbr) for the kernels that walk 32-bit rows.
+  // (ensure_nbr, from t_raw and t_cells) for the kernels that walk 32-bit rows.
   int32_t maxnb = 0;               // capacity of the lists
   bool tile_ok = false, nbr_valid = false;
   int tile_ts = 8;                 // slices per tile
+  int tile_cap = 0;                // places of a tile's search region
   int region = 0;                  // size class of the search region the last rebuild needed
   int64_t ntiles = 0, t_istride = 0, t_entries = 0;
   int32_t t_ustride = 0, tile_umax = 0;
   sph::DBuf<uint16_t> t_idx;       // [nslices][t_istride] union positions x 16
-  sph::DBuf<uint16_t> t_raw;       // [n_pad max_neighbors] places in the tile's search region (scratch)
+  sph::DBuf<uint16_t> t_raw;       // [n_pad max_neighbors] places in the tile's search region, in list order
   sph::DBuf<int2> t_cells;         // [ntiles][kTileCells + 1] (first row, region offset) of the region's cells
   sph::DBuf<int32_t> t_ncell, t_unum, t_uni;   // cells per region, union sizes, unions [ntiles][t_ustride]
   sph::DBuf<int32_t> t_nfl;        // [n_pad] interleaved entries (fluid rows: all; wall rows: the fluid ones)
