@@ -452,8 +452,8 @@ sph_status sph_batch_create(sph_neighbors* const* handles, const sph_visc_params
 sph_status sph_batch_solve(sph_batch* batch, const sph_solve_opts* opts, const double* const* b,
                            double* const* x, sph_solve_report* reports, void* stream);
 
-/* The autotuned persistent-kernel variant (0 when every scene is in the tile form,
- * which has one row loop and 256 threads; else 0..7: row-loop form v & 3 as in
+/* The autotuned persistent-kernel variant (0 where the batch runs on the tile form,
+ * which has one row loop and 256 threads: no other time in tune_ms is set then; else 0..7: row-loop form v & 3 as in
  * sph_profile_counters, block size 256 (v < 4) or 128 threads), whether the
  * solve runs as one graph launch whose conditional WHILE node repeats the pass
  * on the device (2), as a captured pass replayed per pass (1) or as direct

@@ -14,8 +14,9 @@
 // the device which scenes still exceed rtol), pass initialisation, one
 // persistent cooperative kernel that runs all BiCGSTAB iterations of the active
 // scenes with grid barriers between phases, and x += d.  Where every scene has the
-// tile form its applies and residuals run on that (16 scenes, 650k rows: 41.2 ->
-// 36.5 ms a solve); the row-loop forms serve the others.  The whole solve is one
+// tile form and large scenes or long rows prevail (kTileSceneSlices below) its applies
+// and residuals run on that (16 scenes of 10-120k rows: 40.8 -> 36.6 ms a solve); the
+// row-loop forms serve the others.  The whole solve is one
 // CUDA graph launch: the pass sits in the body of a conditional WHILE node whose
 // last kernel decides on the device whether another pass follows (some scene
 // still above rtol, passes left, no barrier timed out); where the driver cannot
@@ -45,11 +46,22 @@ namespace sph {
 constexpr int kTileCands[3] = {16, 32, 64};
 constexpr int kTileDefault = 1;
 constexpr float kTileMargin = 0.97f;
+// When a batch runs on the tile form: when at least half of its rows are in scenes of
+// kTileSceneSlices slices or more (tiles of 8 slices, neighbors.cu) or in scenes of more
+// than kTileSceneEntries entries per row.  A block takes 16 slices in 2 steps with tiles of
+// 8, in 4 or 8 with the smaller tiles of smaller scenes, and each step waits for its union;
+// long rows hide that.  Time over the row loops' (a solve's, per row and iteration), both
+// on one machine, rows of ~75 entries: scenes of 4-30k rows, 3 to 24 of them (46k-349k rows
+// together), 1.20, 1.19, 1.17, 1.22, 1.10, 1.17; of 10-60k, 6 to 20 scenes, 1.13, 1.06, 1.07,
+// 1.00; 12 of 10-80k (a third of the rows in large scenes) 1.08; 20 of 6-90k 1.02; 10 of
+// 15-100k (half) 0.94; 16 of 10-120k 0.92; 3 to 24 of 20-120k 0.94, 0.73, 0.90, 0.88, 0.87.
+// Rows of ~230: 0.87 (3 scenes, 52k rows), 0.86, 0.62, 0.77, 0.75 (10 scenes, 465k).
+constexpr int64_t kTileSceneSlices = 1800;
+constexpr int64_t kTileSceneEntries = 160;
 
-struct SceneDesc {
+// (every phase reads it after a barrier, from L2: what the row loops need comes first)
+struct alignas(128) SceneDesc {
   OpView op;
-  TileView tv;         // the tile form (tiles.cuh), when every scene of the batch has it
-  int32_t ts;          // its slices per tile
   const float* op_lo;
   const double* D64;
   int64_t row_off;     // first row of the scene in the concatenated vectors
@@ -57,7 +69,8 @@ struct SceneDesc {
   int32_t tile_begin, tile_end;
   double bb;           // ||b||^2 of the scene (all components)
   int32_t maxit;
-  int32_t pad;
+  int32_t ts;          // the tile form (tiles.cuh), when the batch runs on it: slices per tile
+  TileView tv;
 };
 
 struct BatchCtrl {
@@ -407,8 +420,10 @@ __global__ void __launch_bounds__(kBlock) kb_init(BatchView B) {
 
 // One BiCGSTAB pass for every active scene: loops over iterations until no
 // scene progresses, with a grid barrier between the phases of an iteration.
+// (0: the compiler's own choice of registers, 56-80 for the row loops; a bound of one block
+// per SM lets it take 100-130, and 2 blocks fit where 3 did: 16% slower at 349k rows)
 template <int U, bool PF, int NB, bool TILE>
-__global__ void __launch_bounds__(NB, TILE ? 4 : 1) kb_pass(BatchView B, int iter_cap) {
+__global__ void __launch_bounds__(NB, TILE ? 4 : 0) kb_pass(BatchView B, int iter_cap) {
   extern __shared__ __align__(16) float4 dyn[];
   __shared__ float part[TILE ? 192 * 3 : 1];
   for (int it = 0; it < iter_cap; ++it) {
@@ -655,7 +670,7 @@ struct sph_batch {
   std::vector<int64_t> row_off;
   std::vector<uint64_t> rs_version;   // each handle's row-scale version at creation
   std::vector<uint64_t> list_version; // and its build count: the tiles, ts and smem below are those lists'
-  bool tile_form = false;             // every scene's operator is in the tile form
+  bool tile_form = false;             // the kernels run on the tile form of every scene's operator
   size_t smem = 0, smem_res = 0;      // dynamic shared memory of the pass and the residual kernels
   DBuf<double> norms;                 // [nscenes][kNormBlocks][3]
   int64_t nrows = 0;
@@ -769,13 +784,12 @@ void scene_view(const sph_batch* Bt, const sph_neighbors* H, SceneDesc& d) {
 }
 
 // Whether a scene's handle still is what the batch was made for: the same lists (the
-// kernels' shared memory and tile sizes are theirs), A(dt) of the scene's parameters in
-// the batch's form, the same row scale.
+// kernels' shared memory and tile sizes are theirs), A(dt) of the scene's parameters, the
+// same row scale.
 bool scene_unchanged(const sph_batch* Bt, int s) {
   const sph_neighbors* H = Bt->handles[s];
   const sph_visc_params& P = Bt->params[s];
-  return H->lists_ok && H->list_version == Bt->list_version[s] && H->op_valid &&
-         (Bt->tile_form ? H->op_tile_valid : H->op_ih_valid) && H->op_mu_version == H->mu_version &&
+  return H->lists_ok && H->list_version == Bt->list_version[s] && H->op_valid && H->op_mu_version == H->mu_version &&
          H->op_params.dt == P.dt && H->op_params.boundary == P.boundary && H->op_params.mean == P.mean &&
          H->rs_version == Bt->rs_version[s] && (!H->row_scaled || H->rs_op_version == H->op_version);
 }
@@ -838,10 +852,15 @@ sph_status sph_batch_create(sph_neighbors* const* handles, const sph_visc_params
   Bt->hdesc.assign(nscenes, SceneDesc{});
   int64_t rows = 0, max_tiles = 0;
   Bt->tile_form = true;
+  int64_t all_rows = 0, tile_rows = 0;
   for (int s = 0; s < nscenes; ++s) {   // (two unions of one-slice tiles have to fit where one does)
     const sph_neighbors* H = handles[s];
     Bt->tile_form = Bt->tile_form && H && H->tile_ok && (H->tile_ts > 1 || 2 * H->tile_umax <= kTileUnion);
+    if (!H) continue;
+    all_rows += H->n;
+    if (H->nslices >= kTileSceneSlices || H->nnz > kTileSceneEntries * H->n) tile_rows += H->n;
   }
+  Bt->tile_form = Bt->tile_form && 2 * tile_rows >= all_rows;
   for (int s = 0; s < nscenes; ++s) {
     sph_neighbors* H = handles[s];
     if (!H) {
@@ -979,7 +998,9 @@ sph_status sph_batch_solve(sph_batch* Bt, const sph_solve_opts* O, const double*
     }
   }
   for (int s = 0; s < S; ++s) {
-    const sph_neighbors* H = Bt->handles[s];
+    sph_neighbors* H = Bt->handles[s];
+    // (a set-up at other parameters and back may have made the other form only)
+    SPH_TRY(ensure_operator(H, &Bt->params[s], st, Bt->tile_form ? OP_FAST : OP_IH));
     scene_view(Bt, H, Bt->hdesc[s]);
     const int64_t o = Bt->row_off[s];
     SPH_LAUNCH(kb_gather, grid_for(H, H->n_pad), kBlock, 0, st)(b[s], H->perm.p, H->n, H->n_pad,
