@@ -40,8 +40,9 @@ namespace sph {
 namespace {
 
 // flags[0]: bits below; [1] largest |coordinate| (bits), [2] fullest cell, [3]
-// largest union
-enum : int32_t { FLAG_NONFINITE = 1, FLAG_CAPACITY = 2, FLAG_BADFIELD = 4, FLAG_REGION = 8 };
+// largest union, [4] largest search region.  FLAG_REGION: a tile's region is larger than
+// the places asked for; FLAG_UNEVEN: a tile's cells are too many for any region size.
+enum : int32_t { FLAG_NONFINITE = 1, FLAG_CAPACITY = 2, FLAG_BADFIELD = 4, FLAG_REGION = 8, FLAG_UNEVEN = 16 };
 
 // a cell this full cannot belong to a particle set of at most maxnb neighbours;
 // the quadratic steps below are not run on one
@@ -392,7 +393,8 @@ __device__ __forceinline__ int tile_entry(int j, int lane) { return (j >> 2) * 1
 // four in turn, list places from a prefix sum over the lanes, so small particle sets
 // still fill the chip.  Entries are places in the region, entry j of a row at
 // rstride * slice + 32 j + lane, in the order of k_neighbors; k_tile_plan turns them
-// into union positions.  A tile that does not fit raises FLAG_REGION and is left.
+// into union positions.  A tile that does not fit raises FLAG_REGION or FLAG_UNEVEN and
+// is left.
 template <int TS, bool PER>
 __global__ void __launch_bounds__(256) k_tile_search(
     const float4* __restrict__ pos_s, const int32_t* __restrict__ key_s, const int32_t* __restrict__ rank,
@@ -476,7 +478,7 @@ __global__ void __launch_bounds__(256) k_tile_search(
   __syncthreads();
   const int m = min(ncell, kTileCells);
   if (nheads > kTileHeads || ncell > kTileCells) {
-    if (tid == 0) atomicOr(&flags[0], FLAG_REGION);
+    if (tid == 0) atomicOr(&flags[0], FLAG_UNEVEN);
     return;
   }
   // cells by rank, and their offsets in the region
@@ -505,6 +507,7 @@ __global__ void __launch_bounds__(256) k_tile_search(
   }
   __syncthreads();
   const int nreg = m > 0 ? soff[m] : 0;
+  if (tid == 0) atomicMax(&flags[4], nreg);
   if (nreg > cap) {
     if (tid == 0) atomicOr(&flags[0], FLAG_REGION);
     return;
@@ -695,7 +698,7 @@ __global__ void __launch_bounds__(256) k_tile_plan(const uint8_t* __restrict__ t
   constexpr unsigned kRef = 0x4000u, kWall = 0x8000u;
   __shared__ int wpre[256];
   __shared__ int wsum[8];
-  if (build_stopped(flags, maxnb) || (flags[0] & (FLAG_REGION | FLAG_CAPACITY)) != 0) return;
+  if (build_stopped(flags, maxnb) || (flags[0] & (FLAG_REGION | FLAG_UNEVEN | FLAG_CAPACITY)) != 0) return;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int64_t tile = blockIdx.x, row0 = tile * R;
   const int2* __restrict__ cells = tcells + tile * (kTileCells + 1);
@@ -996,10 +999,21 @@ sph_status build_slices(sph_neighbors* H, const int32_t* cnt, int64_t* off, int6
 // channels ~3,600, h = 2.5 dp 6,656.  With the first and 128 entries a row three blocks of
 // the plan fit an SM (72.7 KB each; two with 4,608 places); above 160 entries a row it
 // changes nothing and the second comes first.  A handle starts with the size that its
-// last rebuild needed.
+// last rebuild needed (a smaller one only where that leaves a sixteenth free, so that a
+// need that moves about a limit is not searched twice).  A set that no tiles hold is
+// searched globally at once by its next kUntiledRebuilds rebuilds: a dense block under a
+// spray, 54k rows, takes 257 us a rebuild; with failed tile searches each time 634.
 constexpr int kRegions[] = {3584, 4608, 7168};
 constexpr int kRegionSizes = 3;
 constexpr int kRegionLarge = kRegions[kRegionSizes - 1];
+constexpr int kUntiledRebuilds = 32;
+
+// the smallest size class from `least` on with `need` places, kRegionSizes if there is none
+static int region_class(int need, int least) {
+  int k = least;
+  while (k < kRegionSizes && kRegions[k] < need) ++k;
+  return k;
+}
 
 // Slices per tile.  Large tiles share more of their neighbours (4.4 union rows per row
 // at 8 slices, 5.8 at 4, 7.8 at 2 on the box); small ones give a small set more blocks
@@ -1176,6 +1190,8 @@ sph_status build_neighbors(const sph_scene* sc, int32_t maxnb, sph_neighbors** o
   TRYF_CUDA(cudaGetDevice(&H->device));
   TRYF_CUDA(cudaDeviceGetAttribute(&H->num_sms, cudaDevAttrMultiProcessorCount, H->device));
   const int64_t n = sc->n;
+  const bool same_shape = H->n == n && H->h == sc->h && H->kernel == sc->kernel && H->maxnb == maxnb &&
+                          std::equal(g.ncell, g.ncell + 3, H->grid.ncell);
   H->lists_ok = false;
   ++H->list_version;
   if (H->row_scaled && H->n != n) {   // a caller-order row scale no longer fits
@@ -1246,9 +1262,13 @@ sph_status build_neighbors(const sph_scene* sc, int32_t maxnb, sph_neighbors** o
   H->tile_ok = false;
   int32_t hflags[8];
   int64_t tot[2], t_entries = 0;
-  // the tile search with a small region first, with larger ones for the sets that
-  // need it (h = 2.5 dp: 150 particles per cell), then the global scan
-  for (int round = std::max(H->region, maxnb > 160 ? 1 : 0);; ++round) {
+  // the tile search with the region size that the last rebuild needed, once more with
+  // the size that it turns out to need (h = 2.5 dp: 150 particles per cell), then the
+  // global scan
+  if (!same_shape) H->untiled = 0;
+  const int least = maxnb > 160 ? 1 : 0;
+  int round = H->untiled > 0 ? kRegionSizes : std::max(H->region, least);
+  for (;;) {
     const bool tiles = round < kRegionSizes;
     TRYF_CUDA(cudaMemsetAsync(H->tmp_i64.p, 0, 2 * sizeof(int64_t), st));
     if (tiles) {
@@ -1288,10 +1308,12 @@ sph_status build_neighbors(const sph_scene* sc, int32_t maxnb, sph_neighbors** o
       set_error("sph_build_neighbors: non-finite or non-positive density / viscosity");
       return fail(SPH_ERR_NONFINITE);
     }
-    if (tiles && ((hflags[0] & FLAG_REGION) || hflags[3] > kTileUnion)) {
+    if (tiles && ((hflags[0] & (FLAG_REGION | FLAG_UNEVEN)) || hflags[3] > kTileUnion)) {
       TRYF_CUDA(cudaMemsetAsync(H->flags.p, 0, sizeof(int32_t), st));
-      TRYF_CUDA(cudaMemsetAsync(H->flags.p + 3, 0, sizeof(int32_t), st));
-      if (hflags[3] > kTileUnion) round = kRegionSizes - 1;   // a larger region does not help
+      TRYF_CUDA(cudaMemsetAsync(H->flags.p + 3, 0, 2 * sizeof(int32_t), st));
+      const bool larger = !(hflags[0] & FLAG_UNEVEN) && hflags[3] <= kTileUnion;   // whether that helps
+      round = larger ? region_class(hflags[4], round + 1) : kRegionSizes;
+      if (round == kRegionSizes) H->untiled = kUntiledRebuilds + 1;
       continue;
     }
     if (hflags[0] & FLAG_CAPACITY) {
@@ -1300,7 +1322,8 @@ sph_status build_neighbors(const sph_scene* sc, int32_t maxnb, sph_neighbors** o
     }
     H->tile_ok = tiles;
     H->nbr_valid = !tiles;
-    H->region = tiles ? round : 0;
+    if (tiles) H->region = std::min(round, region_class(hflags[4] + hflags[4] / 16, 0));
+    else --H->untiled;
     break;
   }
   H->tile_umax = hflags[3];

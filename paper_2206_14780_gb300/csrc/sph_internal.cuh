@@ -209,7 +209,8 @@ struct sph_neighbors {
   bool tile_ok = false, nbr_valid = false;
   int tile_ts = 8;                 // slices per tile
   int tile_cap = 0;                // places of a tile's search region
-  int region = 0;                  // size class of the search region the last rebuild needed
+  int region = 0;                  // size class of the search region the last tiled rebuild needed
+  int untiled = 0;                 // rebuilds of this shape still to be searched globally at once
   int64_t ntiles = 0, t_istride = 0, t_entries = 0;
   int32_t t_ustride = 0, tile_umax = 0;
   sph::DBuf<uint16_t> t_idx;       // [nslices][t_istride] union positions x 16
