@@ -655,7 +655,10 @@ sph_status sph_set_row_scale(sph_neighbors* handle, const float* scale, void* st
 /* norm2 (device [n] float, caller order) = squared Euclidean norm of each row of
  * D^-1 A(dt) for params: 1 + sum (a / D)^2 over a fluid row's coefficients, 1 +
  * sum S^2 over a dummy-wall row's Shepard weights, 1 for an identity row
- * (float32 sums of the stored float32 coefficients). */
+ * (float32 sums of the stored float32 coefficients).  The first call of this,
+ * sph_wall_row_scale or sph_mlp_scale_targets after a set-up makes the coefficients
+ * along 32-bit rows: it allocates and synchronises, so it comes before a stream
+ * capture of one. */
 sph_status sph_row_norms(sph_neighbors* handle, const sph_visc_params* params, float* norm2, void* stream);
 
 /* The closed-form wall scale: scale (device [n] float, caller order) =

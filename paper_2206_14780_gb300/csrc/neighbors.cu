@@ -1051,6 +1051,11 @@ sph_status require_lists(const sph_neighbors* H) {
   return SPH_ERR_INVALID;
 }
 
+bool stream_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(st, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone;
+}
+
 sph_status ensure_nbr(sph_neighbors* H, cudaStream_t st) {
   SPH_TRY(require_lists(H));
   if (H->nbr_valid) return SPH_OK;
@@ -1059,6 +1064,8 @@ sph_status ensure_nbr(sph_neighbors* H, cudaStream_t st) {
   SPH_LAUNCH(k_tile_expand, (int)H->ntiles, 256, H->tile_cap * sizeof(int32_t), st)(
       H->t_raw.p, H->t_cells.p, H->t_ncell.p, H->cnt.p, H->tile_ts, H->nslices, H->n, H->maxnb, H->nbr.p);
   SPH_TRY_CUDA(cudaGetLastError());
+  if (stream_capturing(st)) return SPH_OK;
+  SPH_TRY_CUDA(cudaStreamSynchronize(st));
   H->nbr_valid = true;
   return SPH_OK;
 }

@@ -363,6 +363,10 @@ sph_status ensure_operator(sph_neighbors* H, const sph_visc_params* P, cudaStrea
   const bool same = H->op_valid && H->op_params.dt == P->dt && H->op_params.boundary == P->boundary &&
                     H->op_params.mean == P->mean && H->op_mu_version == H->mu_version;
   if (same && (tile ? H->op_tile_valid : H->op_ih_valid)) return SPH_OK;
+  if (stream_capturing(st)) {   // it would count as set up before anything has run
+    set_error("the coefficients for these parameters are not set up, and the stream is capturing: call before the capture");
+    return SPH_ERR_CUDA;
+  }
   if (!same) {
     H->op_valid = H->op_tile_valid = H->op_ih_valid = false;
     ++H->op_version;

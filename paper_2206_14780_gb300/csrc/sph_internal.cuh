@@ -339,7 +339,10 @@ namespace sph {
 // neighbors.cu
 // SPH_ERR_INVALID while the handle's last build has not succeeded
 sph_status require_lists(const sph_neighbors* H);
-// the 32-bit rows of the lists (nbr, slice_off), expanded from the tiles if need be
+bool stream_capturing(cudaStream_t st);
+// the 32-bit rows of the lists (nbr, slice_off), expanded from the tiles if need be:
+// complete on return, as lists are after a build, so calls on any stream may read them;
+// while the stream is capturing they become part of the graph and stay to be made outside
 sph_status ensure_nbr(sph_neighbors* H, cudaStream_t st);
 
 sph_status build_slices(sph_neighbors* H, const int32_t* cnt, int64_t* off, int64_t* total_pad, int64_t* total,
