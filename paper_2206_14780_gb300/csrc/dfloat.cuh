@@ -2,16 +2,10 @@
 // (Knuth's TwoSum; Dekker's TwoProd through fma).
 #pragma once
 
+#include "exact_sum.cuh"
 #include "sph_internal.cuh"
 
 namespace sph {
-
-// Knuth's TwoSum: s + e == a + b exactly (no branch, any magnitudes)
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  const float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
-}
 
 // sum_a a_ba (kap x_b - x_a) for one component with float32 error-free
 // transformations: the difference of the hi parts exactly (TwoSum), its product

@@ -23,6 +23,7 @@
 // velocity.  Position and density updates are evaluated in float64 with one
 // rounding per operation (no contraction) and stored as float32, so the half
 // step's positions -- and hence its neighbour lists -- are reproducible.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -210,8 +211,8 @@ __global__ void __launch_bounds__(kBlock) k_step_forces(const float4* __restrict
 // k_step_dummy and k_step_forces walk the 32-bit lists with one thread per row and add
 // in float64 (63 cycles an addition and a conversion): 85 and 149 us on 91k rows, 47
 // and 70 us on 1.4k.  Here the union's data come from shared memory, S = 8 / TS threads
-// share a row, and the sums run in double-float arithmetic (TwoSum; a few 2^-47 of the
-// terms' magnitudes, stored to float32 as before).
+// share a row, and the sums run in three float32 parts (Sum3: closer than a float64 sum;
+// stored to float32 as before).
 
 struct TileLists {
   const uint16_t* idx;
@@ -226,33 +227,30 @@ TileLists tile_lists(const sph_neighbors* H) {
                    H->cnt.p,    H->t_ustride, (int32_t)H->ntiles, H->nslices};
 }
 
-// running sum: s + e follows the exact sum of the terms
-struct Sum2 {
-  float s = 0.f, e = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    float t, r;
-    two_sum(s, x, t, r);
-    s = t;
-    e += r;
-  }
-  __device__ __forceinline__ void add(const Sum2& o) {
-    add(o.s);
-    e += o.e;
-  }
-  __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+// the scales k_tile_dummy works in, powers of two: with them the weights, pressures and
+// densities are near one whatever the units are (weights near 2^40 at the centre, so that
+// the small ones near the support's edge lose nothing either), and no product leaves
+// float32's range where the float64 sums stay in theirs
+struct DummyScales {
+  float p, rho;          // factors of pressures and densities
+  double P, gr;          // of the sums' two parts
 };
 
-// dummy walls, as k_step_dummy
+// Dummy walls, as k_step_dummy: sum w (P + g.r rho) as sum w P + g . sum (w rho r), each
+// product exact.  geo.w_scale: the kernel's constant in the scale above (it cancels in
+// P_w).
 template <int TS>
 __global__ void __launch_bounds__(256) k_tile_dummy(TileLists L, const float4* __restrict__ pos_s, float* rho_s,
                                                     const uint8_t* __restrict__ type_s, const int32_t* __restrict__ perm,
-                                                    int64_t n, StepGeom g, dfl gx, dfl gy, dfl gz, double rho0, double c0,
-                                                    Zeta zeta, float* P_s, float* __restrict__ rho_c) {
+                                                    int64_t n, StepGeom geo, DummyScales sc, double gx, double gy,
+                                                    double gz, double rho0, double c0, Zeta zeta, float* P_s,
+                                                    float* __restrict__ rho_c) {
   constexpr int S = 8 / TS, R = 32 * TS;
   extern __shared__ __align__(16) float4 dyn[];
-  __shared__ float part[S > 1 ? S - 1 : 1][4][R];
+  __shared__ float part[S > 1 ? S - 1 : 1][15][R];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int split = wid / TS, row = (wid % TS) * 32 + lane;
+  const bool on[3] = {gx != 0.0, gy != 0.0, gz != 0.0};
   for (int64_t tile = blockIdx.x; tile < L.ntiles; tile += gridDim.x) {
     const int64_t sl = tile * TS + wid % TS, s = sl * kSlice + lane;
     const bool wall = s < n && type_s[s] != SPH_FLUID;
@@ -264,40 +262,44 @@ __global__ void __launch_bounds__(256) k_tile_dummy(TileLists L, const float4* _
       const int t = ids[i];
       if (type_s[t] != SPH_FLUID) continue;   // walls are being rewritten; no row reads them
       X[i] = pos_s[t];
-      Y[i] = make_float4(P_s[t], rho_s[t], 0.f, 0.f);
+      Y[i] = make_float4(P_s[t] * sc.p, rho_s[t] * sc.rho, 0.f, 0.f);
     }
     __syncthreads();
     const int nf = wall ? L.nfl[s] : 0;
     const float4 pb = wall ? pos_s[s] : make_float4(0.f, 0.f, 0.f, 0.f);
-    Sum2 W;
-    dfl num{0.f, 0.f};
+    Sum3 sum[5];   // w, w P, w rho r
     tile_walk(L.idx, L.istride, sl, lane, nf, nf, split, S, [&](uint32_t o) {
       const float4 pa = tile_at(X, o), q4 = tile_at(Y, o);
       float d[3] = {pb.x - pa.x, pb.y - pa.y, pb.z - pa.z};   // r_w - r_a
-      min_image(d, g);
-      const float w = kernel_w(sqrtf(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]) * g.inv_h, g);
-      const dfl gr = df_add(df_add(df_mul(gx, dfl{d[0], 0.f}), df_mul(gy, dfl{d[1], 0.f})), df_mul(gz, dfl{d[2], 0.f}));
-      W.add(w);
-      num = df_add(num, df_mul(dfl{w, 0.f}, df_add(dfl{q4.x, 0.f}, df_mul(gr, dfl{q4.y, 0.f}))));
+      min_image(d, geo);
+      const float w = kernel_w(sqrtf(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]) * geo.inv_h, geo);
+      sum[0].add(w);
+      sum[1].add_product(w, q4.x);
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        if (on[k]) sum[2 + k].add_product(w, q4.y, d[k]);
     });
     if (S > 1) {
       if (split > 0) {
         float(*q)[R] = part[split - 1];
-        q[0][row] = W.s;
-        q[1][row] = W.e;
-        q[2][row] = num.hi;
-        q[3][row] = num.lo;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          q[3 * k][row] = sum[k].s;
+          q[3 * k + 1][row] = sum[k].e;
+          q[3 * k + 2][row] = sum[k].f;
+        }
       }
       __syncthreads();
       if (split == 0)
-        for (int k = 0; k < S - 1; ++k) {
-          W.add(Sum2{part[k][0][row], part[k][1][row]});
-          num = df_add(num, dfl{part[k][2][row], part[k][3][row]});
+        for (int w = 0; w < S - 1; ++w) {
+#pragma unroll
+          for (int k = 0; k < 5; ++k) sum[k].add(Sum3{part[w][3 * k][row], part[w][3 * k + 1][row], part[w][3 * k + 2][row]});
         }
     }
     if (wall && split == 0) {
-      const double Sw = W.value();
-      const double P = Sw > 0.0 ? df_to_double(num) / Sw : 0.0;
+      const double Sw = sum[0].value();
+      const double gr = gx * sum[2].value() + gy * sum[3].value() + gz * sum[4].value();
+      const double P = Sw > 0.0 ? (sc.P * sum[1].value() + sc.gr * gr) / Sw : 0.0;
       const double r = rho0 * zeta_root(P * zeta.z / (c0 * c0 * rho0) + 1.0, zeta);
       P_s[s] = (float)P;
       rho_s[s] = (float)r;
@@ -317,7 +319,7 @@ __global__ void __launch_bounds__(256) k_tile_forces(TileLists L, const float4* 
                                                      float* __restrict__ drho) {
   constexpr int S = 8 / TS, R = 32 * TS;
   extern __shared__ __align__(16) float4 dyn[];
-  __shared__ float part[S > 1 ? S - 1 : 1][8][R];
+  __shared__ float part[S > 1 ? S - 1 : 1][12][R];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int split = wid / TS, row = (wid % TS) * 32 + lane;
   for (int64_t tile = blockIdx.x; tile < L.ntiles; tile += gridDim.x) {
@@ -349,7 +351,7 @@ __global__ void __launch_bounds__(256) k_tile_forces(TileLists L, const float4* 
       Pb = P_s[s] / (rb * rb);
     }
     __syncthreads();
-    Sum2 ax, ay, az, dr;
+    Sum3 sum[4];   // abar, drho
     tile_walk(L.idx, L.istride, sl, lane, nf, c, split, S, [&](uint32_t o) {
       const float4 pa = tile_at(X, o), ua = tile_at(Y, o);
       float d[3] = {pa.x - pb.x, pa.y - pb.y, pa.z - pb.z};   // r_a - r_b
@@ -357,36 +359,32 @@ __global__ void __launch_bounds__(256) k_tile_forces(TileLists L, const float4* 
       const float q = sqrtf(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]) * g.inv_h;
       const float mF = pa.w * kernel_absf(q, g);
       const float cp = mF * (ua.w + Pb);
-      ax.add(-(cp * d[0]));
-      ay.add(-(cp * d[1]));
-      az.add(-(cp * d[2]));
-      dr.add(mF * ((ub.x - ua.x) * d[0] + (ub.y - ua.y) * d[1] + (ub.z - ua.z) * d[2]));
+#pragma unroll
+      for (int k = 0; k < 3; ++k) sum[k].add(-(cp * d[k]));
+      sum[3].add(mF * ((ub.x - ua.x) * d[0] + (ub.y - ua.y) * d[1] + (ub.z - ua.z) * d[2]));
     });
     if (S > 1) {
       if (split > 0) {
         float(*q)[R] = part[split - 1];
-        q[0][row] = ax.s;
-        q[1][row] = ax.e;
-        q[2][row] = ay.s;
-        q[3][row] = ay.e;
-        q[4][row] = az.s;
-        q[5][row] = az.e;
-        q[6][row] = dr.s;
-        q[7][row] = dr.e;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          q[3 * k][row] = sum[k].s;
+          q[3 * k + 1][row] = sum[k].e;
+          q[3 * k + 2][row] = sum[k].f;
+        }
       }
       __syncthreads();
       if (split == 0)
-        for (int k = 0; k < S - 1; ++k) {
-          ax.add(Sum2{part[k][0][row], part[k][1][row]});
-          ay.add(Sum2{part[k][2][row], part[k][3][row]});
-          az.add(Sum2{part[k][4][row], part[k][5][row]});
-          dr.add(Sum2{part[k][6][row], part[k][7][row]});
+        for (int w = 0; w < S - 1; ++w) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) sum[k].add(Sum3{part[w][3 * k][row], part[w][3 * k + 1][row], part[w][3 * k + 2][row]});
         }
     }
     if (live && split == 0) {
-      acc[ib] = fluid ? make_float4((float)(ax.value() + gx), (float)(ay.value() + gy), (float)(az.value() + gz), 0.f)
+      acc[ib] = fluid ? make_float4((float)(sum[0].value() + gx), (float)(sum[1].value() + gy),
+                                    (float)(sum[2].value() + gz), 0.f)
                       : make_float4(0.f, 0.f, 0.f, 0.f);
-      drho[ib] = on ? (float)dr.value() : 0.f;
+      drho[ib] = on ? (float)sum[3].value() : 0.f;
     }
     __syncthreads();
   }
@@ -474,6 +472,12 @@ __global__ void k_step_change(const double* __restrict__ x, const double* __rest
   }
 }
 
+// the constant of W(q): its value over h^3
+double w_constant(const sph_neighbors* H) {
+  const double h = (double)H->h;
+  return (H->kernel == SPH_KERNEL_GAUSSIAN ? 1.0 / gauss_norm() : 21.0 / (16.0 * M_PI)) / (h * h * h);
+}
+
 StepGeom step_geom(const sph_neighbors* H, const sph_state* S) {
   StepGeom g{};
   for (int ax = 0; ax < 3; ++ax) {
@@ -488,9 +492,22 @@ StepGeom step_geom(const sph_neighbors* H, const sph_state* S) {
   g.gauss = H->kernel == SPH_KERNEL_GAUSSIAN ? 1 : 0;
   const double wg = gauss_norm();
   g.absf_scale = (float)((g.gauss ? 2.0 / wg : 105.0 / (128.0 * M_PI)) / (h * h * h * h * h));
-  g.w_scale = (float)((g.gauss ? 1.0 / wg : 21.0 / (16.0 * M_PI)) / (h * h * h));
+  g.w_scale = (float)w_constant(H);
   g.gauss_tail = (float)std::exp(-kGaussK * kGaussK);
   return g;
+}
+
+// DummyScales for a step, and the kernel's constant in gw (the same float32 mantissa)
+DummyScales dummy_scales(const sph_neighbors* H, const sph_step_params* P, StepGeom& gw) {
+  auto exponent = [](double x) {
+    int e = 0;
+    if (x > 0.0 && std::isfinite(x)) std::frexp(x, &e);
+    return std::min(std::max(e, -120), 120);
+  };
+  const int ep = exponent(P->c0 * P->c0 * P->rho0 / P->zeta), er = exponent(P->rho0);
+  int ew = 0;
+  gw.w_scale = (float)std::ldexp(std::frexp(w_constant(H), &ew), 40);
+  return DummyScales{(float)std::ldexp(1.0, -ep), (float)std::ldexp(1.0, -er), std::ldexp(1.0, ep), std::ldexp(1.0, er)};
 }
 
 sph_scene scene_of(const sph_state* S) {
@@ -531,16 +548,14 @@ sph_status evaluate(sph_state* S, const sph_step_params* Pp, sph_neighbors** han
   const int dummy = Pp->boundary == SPH_BC_DUMMY ? 1 : 0;
   const float4* vel = reinterpret_cast<const float4*>(S->vel);
   const size_t smem = tile_smem(H, 32);
-  auto split = [](double x) {
-    const float hi = (float)x;
-    return dfl{hi, (float)(x - (double)hi)};
-  };
   if (dummy) {
     if (H->tile_ok) {
       auto kern = SPH_TILE_PICK(H, k_tile_dummy);
+      StepGeom gw = g;
+      const DummyScales sc = dummy_scales(H, Pp, gw);
       SPH_LAUNCH(kern, tile_grid(H, (const void*)kern, smem), 256, smem, st)(
-          tile_lists(H), H->pos_s.p, H->rho_s.p, H->type_s.p, H->perm.p, H->n, g, split(Pp->g[0]), split(Pp->g[1]),
-          split(Pp->g[2]), Pp->rho0, Pp->c0, zeta, T.P_s.p, S->rho);
+          tile_lists(H), H->pos_s.p, H->rho_s.p, H->type_s.p, H->perm.p, H->n, gw, sc, Pp->g[0], Pp->g[1], Pp->g[2],
+          Pp->rho0, Pp->c0, zeta, T.P_s.p, S->rho);
     } else {
       SPH_LAUNCH(k_step_dummy, grid, kBlock, 0, st)(H->pos_s.p, H->rho_s.p, H->type_s.p, H->cnt.p, H->slice_off.p,
                                                      H->nbr.p, H->perm.p, H->n, g, Pp->g[0], Pp->g[1], Pp->g[2],
