@@ -203,6 +203,7 @@ sph_status sph_neighbors_destroy(sph_neighbors* h) {
   for (auto& e : h->sa_ev)
     if (e) cudaEventDestroy(e);
   h->persist_buf.release();
+  if (h->nbr_event) cudaEventDestroy(h->nbr_event);
   if (h->host_persist) cudaFreeHost(h->host_persist);
   if (h->host_scal) cudaFreeHost(h->host_scal);
   if (h->host_flags) cudaFreeHost(h->host_flags);

@@ -1058,14 +1058,21 @@ bool stream_capturing(cudaStream_t st) {
 
 sph_status ensure_nbr(sph_neighbors* H, cudaStream_t st) {
   SPH_TRY(require_lists(H));
-  if (H->nbr_valid) return SPH_OK;
+  if (H->nbr_ready) return SPH_OK;
+  const bool capturing = stream_capturing(st);
+  if (H->nbr_valid && !capturing) {   // expanded by an earlier call, on whatever stream
+    if (cudaEventQuery(H->nbr_event) == cudaSuccess) H->nbr_ready = true;
+    else SPH_TRY_CUDA(cudaStreamWaitEvent(st, H->nbr_event, 0));
+    return SPH_OK;
+  }
   SPH_TRY(H->nbr.alloc(H->n_pad * (int64_t)H->maxnb));
   SPH_TRY(fixed_offsets(H, st));
   SPH_LAUNCH(k_tile_expand, (int)H->ntiles, 256, H->tile_cap * sizeof(int32_t), st)(
       H->t_raw.p, H->t_cells.p, H->t_ncell.p, H->cnt.p, H->tile_ts, H->nslices, H->n, H->maxnb, H->nbr.p);
   SPH_TRY_CUDA(cudaGetLastError());
-  if (stream_capturing(st)) return SPH_OK;
-  SPH_TRY_CUDA(cudaStreamSynchronize(st));
+  if (capturing) return SPH_OK;
+  if (!H->nbr_event) SPH_TRY_CUDA(cudaEventCreateWithFlags(&H->nbr_event, cudaEventDisableTiming));
+  SPH_TRY_CUDA(cudaEventRecord(H->nbr_event, st));
   H->nbr_valid = true;
   return SPH_OK;
 }
@@ -1265,7 +1272,7 @@ sph_status build_neighbors(const sph_scene* sc, int32_t maxnb, sph_neighbors** o
   }
 
   H->maxnb = maxnb;
-  H->nbr_valid = false;
+  H->nbr_valid = H->nbr_ready = false;
   H->tile_ok = false;
   int32_t hflags[8];
   int64_t tot[2], t_entries = 0;
@@ -1328,7 +1335,7 @@ sph_status build_neighbors(const sph_scene* sc, int32_t maxnb, sph_neighbors** o
       return fail(SPH_ERR_CAPACITY);
     }
     H->tile_ok = tiles;
-    H->nbr_valid = !tiles;
+    H->nbr_valid = H->nbr_ready = !tiles;
     if (tiles) H->region = std::min(round, region_class(hflags[4] + hflags[4] / 16, 0));
     else --H->untiled;
     break;

@@ -206,7 +206,9 @@ struct sph_neighbors {
   // particle set allows it (tile_ok); nbr and slice_off are then made on demand
   // (ensure_nbr, from t_raw and t_cells) for the kernels that walk 32-bit rows.
   int32_t maxnb = 0;               // capacity of the lists
-  bool tile_ok = false, nbr_valid = false;
+  bool tile_ok = false;
+  bool nbr_valid = false, nbr_ready = false;   // nbr has been enqueued (done at nbr_event); is complete
+  cudaEvent_t nbr_event = nullptr;
   int tile_ts = 8;                 // slices per tile
   int tile_cap = 0;                // places of a tile's search region
   int region = 0;                  // size class of the search region the last tiled rebuild needed
@@ -340,9 +342,10 @@ namespace sph {
 // SPH_ERR_INVALID while the handle's last build has not succeeded
 sph_status require_lists(const sph_neighbors* H);
 bool stream_capturing(cudaStream_t st);
-// the 32-bit rows of the lists (nbr, slice_off), expanded from the tiles if need be:
-// complete on return, as lists are after a build, so calls on any stream may read them;
-// while the stream is capturing they become part of the graph and stay to be made outside
+// the 32-bit rows of the lists (nbr, slice_off), expanded from the tiles if need be: made
+// before what is enqueued on st next, also where another stream expanded them.  While st
+// is capturing the expansion becomes part of the graph (unless the rows are known to be
+// complete) and does not count as made outside.
 sph_status ensure_nbr(sph_neighbors* H, cudaStream_t st);
 
 sph_status build_slices(sph_neighbors* H, const int32_t* cnt, int64_t* off, int64_t* total_pad, int64_t* total,
