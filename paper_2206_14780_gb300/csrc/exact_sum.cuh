@@ -12,11 +12,23 @@
 
 namespace sph {
 
+// one rounded operation, never merged with another into a multiply-add (a host build of
+// this file needs -ffp-contract=off)
+#ifdef __CUDA_ARCH__
+SPH_HD float add_rn(float a, float b) { return __fadd_rn(a, b); }
+SPH_HD float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+SPH_HD double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+#else
+SPH_HD float add_rn(float a, float b) { return a + b; }
+SPH_HD float mul_rn(float a, float b) { return a * b; }
+SPH_HD double mul_rn(double a, double b) { return a * b; }
+#endif
+
 // Knuth's TwoSum: s + e == a + b exactly (no branch, any magnitudes)
 SPH_HD void two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  const float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
+  s = add_rn(a, b);
+  const float bb = add_rn(s, -a);
+  e = add_rn(add_rn(a, -add_rn(s, -bb)), add_rn(b, -bb));
 }
 
 // A running sum in three float32 parts, s + e + f: the rounding errors of s are added
@@ -40,13 +52,13 @@ struct Sum3 {
   }
   // a b, exactly: the product and its rounding error
   SPH_HD void add_product(float a, float b) {
-    const float p = a * b;
+    const float p = mul_rn(a, b);
     add(p);
     add_low(fmaf(a, b, -p));
   }
   // a b c, exactly: (p + q) c with p + q = a b
   SPH_HD void add_product(float a, float b, float c) {
-    const float p = a * b, q = fmaf(a, b, -p), t = p * c, u = q * c;
+    const float p = mul_rn(a, b), q = fmaf(a, b, -p), t = mul_rn(p, c), u = mul_rn(q, c);
     add(t);
     add_low(fmaf(p, c, -t));
     add_low(u);
