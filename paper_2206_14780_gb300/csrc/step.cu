@@ -30,6 +30,7 @@
 #include "dfloat.cuh"
 #include "sph_internal.cuh"
 #include "tiles.cuh"
+#include "whole_power.cuh"
 
 namespace sph {
 
@@ -95,29 +96,23 @@ __device__ __forceinline__ float kernel_w(float q, const StepGeom& g) {
 
 // The equation of state's exponent: zeta itself, and k = zeta where that is a whole
 // number from 2 to 16 (7 for water), else 0.  A float64 instruction costs a warp ~63
-// cycles and pow over a hundred of them; x^k by squaring is 4 at k = 7, and the root one
-// Halley step from the float32 root (error (k^2 - 1) / 12 e^3 of its ~3e-7), both within
-// a few units of float64's last place before the result is rounded to float32.  The
-// pressures of 91k rows took 26 us with pow, the walls' 37 us are 29 us with the root.
+// cycles and pow over a hundred of them; x^k by squaring with its rounding errors
+// carried along is ~20 at k = 7 and the root one step from the float32 root
+// (whole_power.cuh: both within 0.52 units of float64's last place).  The pressures of
+// 91k rows take 14 us, 26 with pow (8 with plain squaring, up to 5 units off).
 struct Zeta {
   double z;
   int k;
 };
 Zeta make_zeta(double z) { return Zeta{z, z >= 2.0 && z <= 16.0 && z == std::floor(z) ? (int)z : 0}; }
 
-__device__ __forceinline__ double whole_pow(double x, int k) {
-  double r = (k & 1) ? x : 1.0;
-  for (k >>= 1; k > 0; k >>= 1) {
-    x *= x;
-    if (k & 1) r *= x;
-  }
-  return r;
+// x^zeta - 1
+__device__ __forceinline__ double zeta_pow_m1(double x, Zeta e) {
+  return e.k ? whole_pow_m1(x, e.k) : pow(x, e.z) - 1.0;
 }
-__device__ __forceinline__ double zeta_pow(double x, Zeta e) { return e.k ? whole_pow(x, e.k) : pow(x, e.z); }
 __device__ __forceinline__ double zeta_root(double v, Zeta e) {
   if (e.k == 0 || !(v > 1e-30 && v < 1e30)) return pow(v, 1.0 / e.z);
-  const double y = (double)powf((float)v, 1.f / (float)e.k), p = whole_pow(y, e.k);
-  return y + y * (2.0 * (v - p)) / ((double)(e.k + 1) * p + (double)(e.k - 1) * v);
+  return whole_root(v, e.k);
 }
 
 // P = EOS(rho) on every sorted row (dummy walls are overwritten by the closure)
@@ -125,7 +120,7 @@ __global__ void k_step_eos(const float* __restrict__ rho_s, int64_t n, double rh
                            float* __restrict__ P_s) {
   const double scale = c0 * c0 * rho0 / zeta.z;
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x)
-    P_s[s] = (float)(scale * (zeta_pow((double)rho_s[s] / rho0, zeta) - 1.0));
+    P_s[s] = (float)(scale * zeta_pow_m1((double)rho_s[s] / rho0, zeta));
 }
 
 // dummy walls (Eq. dummyP): pressure from the fluid neighbours, density by the
@@ -212,7 +207,7 @@ __global__ void __launch_bounds__(kBlock) k_step_forces(const float4* __restrict
 // in float64 (63 cycles an addition and a conversion): 85 and 149 us on 91k rows, 47
 // and 70 us on 1.4k.  Here the union's data come from shared memory, S = 8 / TS threads
 // share a row, and the sums run in three float32 parts (Sum3: closer than a float64 sum;
-// stored to float32 as before).
+// stored to float32 as before): 42 and 48 us on 91k rows.
 
 struct TileLists {
   const uint16_t* idx;
