@@ -82,6 +82,17 @@ __device__ __forceinline__ dfl df_rcp(dfl a) {
   const float r = fmaf(-a.lo, y, fmaf(-a.hi, y, 1.f));
   return df_quick(y, y * r);
 }
+// a / b in double-float, a = hi + lo, for a.hi, b > 0: the remainder of the rounded quotient
+// is exact in one fma, so the error is the low quotient's rounding (2^-48).  Worked out on
+// the mantissas and scaled back, so that nothing is lost at either end of float32's range
+// while the quotient is inside it; times 2^scale.
+__device__ __forceinline__ dfl df_quotient(dfl a, float b, int scale = 0) {
+  int ea, eb;
+  const float ah = frexpf(a.hi, &ea), bm = frexpf(b, &eb), al = scalbnf(a.lo, -ea);
+  const float q = __fdiv_rn(ah, bm);
+  const dfl r = df_quick(q, __fdiv_rn(fmaf(-q, bm, ah) + al, bm));
+  return dfl{scalbnf(r.hi, ea - eb + scale), scalbnf(r.lo, ea - eb + scale)};
+}
 __device__ __forceinline__ dfl df_from_double(double x) {
   const float hi = __double2float_rn(x);
   return dfl{hi, __double2float_rn(x - (double)hi)};

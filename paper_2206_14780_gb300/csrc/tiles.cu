@@ -34,13 +34,12 @@ int tile_grid(const sph_neighbors* H, const void* kernel, size_t smem) {
 namespace {
 
 // per particle: V = m / rho and 1 / mu as double-float pairs (V hi, V lo, 1/mu hi,
-// 1/mu lo): the remainder of a correctly rounded quotient is exact in one fma
+// 1/mu lo)
 __global__ void k_tile_aux(const float4* __restrict__ pos, const float* __restrict__ rho, const float* __restrict__ mu,
                            int64_t n_pad, float4* __restrict__ aux) {
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_pad; s += (int64_t)gridDim.x * blockDim.x) {
-    const float m = pos[s].w, r = rho[s], u = mu[s];
-    const float v = __fdiv_rn(m, r), w = __frcp_rn(u);
-    aux[s] = make_float4(v, __fdiv_rn(fmaf(-v, r, m), r), w, __fdiv_rn(fmaf(-w, u, 1.f), u));
+    const dfl v = df_quotient(dfl{pos[s].w, 0.f}, rho[s]), w = df_quotient(dfl{1.f, 0.f}, mu[s]);
+    aux[s] = make_float4(v.hi, v.lo, w.hi, w.lo);
   }
 }
 
@@ -53,7 +52,8 @@ struct FillArgs {
   const int32_t* nfl;
   int64_t n;
   OpGeomDF g;
-  dfl kf;              // 2 dt times the constant of |f| over h^5
+  dfl kf;              // 2 dt times the constant of |f| over h^5, divided by 2^kf_exp
+  int kf_exp;
   int dummy, arithmetic, gauss;
   dfl gauss_tail;      // e^{-9}
   float* hi;
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(256) k_tile_fill(TileView op, FillArgs A) {
       const float mu_b = A.mu[s];
       const float4 ab = A.aux[s];
       const dfl imu_b{ab.z, ab.w};
-      const dfl Rb = c > 0 ? df_mul(A.kf, df_rcp(dfl{A.rho[s], 0.f})) : dfl{0.f, 0.f};
+      const dfl Rb = c > 0 ? df_quotient(A.kf, A.rho[s], A.kf_exp) : dfl{0.f, 0.f};
       for (int g = split; g < ng; g += S) {
         uint32_t o[4];
         tile_unpack(pi[g * 32], o);
@@ -411,7 +411,8 @@ sph_status tile_fill(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st
   A.g.inv_h = split(ih);
   A.g.inv_h2 = split(ih * ih);
   A.gauss = H->kernel == SPH_KERNEL_GAUSSIAN ? 1 : 0;
-  A.kf = split(2.0 * P->dt * (A.gauss ? 2.0 / gauss_norm() : 105.0 / (128.0 * M_PI)) * (ih * ih * ih * ih * ih));
+  A.kf = split(std::frexp(2.0 * P->dt * (A.gauss ? 2.0 / gauss_norm() : 105.0 / (128.0 * M_PI)) * (ih * ih * ih * ih * ih),
+                          &A.kf_exp));
   A.pos = H->pos_s.p;
   A.rho = H->rho_s.p;
   A.mu = H->mu_s.p;
