@@ -449,16 +449,16 @@ __global__ void __launch_bounds__(kPT, 1) k_persist(PersistArgs A) {
     for (int i = tid; i < U; i += kPT) P[i] = __ldcg(A.d + ID[i]);
     __syncthreads();
     double sums[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    auto finish64 = [&](int r, const float* v) {
+    auto finish64 = [&](int r, const double (&v)[3]) {
       const int64_t s = row0 + r;
       const unsigned kd = info[r] >> 16;
       const double sg = kd == KIND_FLUID ? 1.0 : (kd == KIND_SHEPARD ? -1.0 : 0.0);
       const float4 db = __ldcg(A.d + s);
       double r0 = 0.0, r1 = 0.0, r2 = 0.0;
       if (s < A.n) {
-        r0 = A.r64[3 * s] - ((double)db.x + sg * ((double)v[0] + (double)v[1]));
-        r1 = A.r64[3 * s + 1] - ((double)db.y + sg * ((double)v[2] + (double)v[3]));
-        r2 = A.r64[3 * s + 2] - ((double)db.z + sg * ((double)v[4] + (double)v[5]));
+        r0 = A.r64[3 * s] - ((double)db.x + sg * v[0]);
+        r1 = A.r64[3 * s + 1] - ((double)db.y + sg * v[1]);
+        r2 = A.r64[3 * s + 2] - ((double)db.z + sg * v[2]);
       }
       A.r64[3 * s] = r0;
       A.r64[3 * s + 1] = r1;
@@ -479,33 +479,29 @@ __global__ void __launch_bounds__(kPT, 1) k_persist(PersistArgs A) {
         tile_residual_row<false>(op, X, X, sl0 + i, lane, (int)(in & 0xffffu), split, SP,
                                  make_float4(kap * db.x, kap * db.y, kap * db.z, 0.f),
                                  make_float4(0.f, 0.f, 0.f, 0.f), x0, x1, x2);
-      const float v[6] = {x0.sh, x0.sl + x0.c, x1.sh, x1.sl + x1.c, x2.sh, x2.sl + x2.c};
       if (SP == 1) {
-        finish64(r, v);
+        finish64(r, {x0.value(), x1.value(), x2.value()});
       } else {
+        const SplitSum v[3] = {SplitSum(x0), SplitSum(x1), SplitSum(x2)};
         float* q = part + ((size_t)split * NR + r) * 6;
 #pragma unroll
-        for (int k = 0; k < 6; ++k) q[k] = v[k];
+        for (int k = 0; k < 3; ++k) {
+          q[2 * k] = v[k].hi;
+          q[2 * k + 1] = v[k].lo;
+        }
       }
     }
     if (SP > 1) {
       __syncthreads();
       for (int r = tid; r < NR; r += kPT) {
-        float v[6];
         const float* q = part + (size_t)r * 6;
-#pragma unroll
-        for (int k = 0; k < 6; ++k) v[k] = q[k];
-        for (int w = 1; w < SP; ++w) {   // the splits' sums, their high parts exactly
+        SplitSum v[3] = {SplitSum(q[0], q[1]), SplitSum(q[2], q[3]), SplitSum(q[4], q[5])};
+        for (int w = 1; w < SP; ++w) {
           q += (size_t)NR * 6;
 #pragma unroll
-          for (int k = 0; k < 6; k += 2) {
-            float t, e;
-            two_sum(v[k], q[k], t, e);
-            v[k] = t;
-            v[k + 1] += q[k + 1] + e;
-          }
+          for (int k = 0; k < 3; ++k) v[k].add(SplitSum(q[2 * k], q[2 * k + 1]));
         }
-        finish64(r, v);
+        finish64(r, {v[0].value(), v[1].value(), v[2].value()});
       }
     }
     // (this barrier also holds the next pass's reset of d back until every block has

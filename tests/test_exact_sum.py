@@ -16,6 +16,35 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 OUT = os.path.join(ROOT, "paper_2206_14780_gb300", "_build", "exact_sum_probe")
 
+# rows of a residual: n terms a (k - x), a and x given as (a hi, a lo, x), one accumulator, or
+# `splits` of them taking groups of four terms in turn and put together as the solve does
+ROWS = r"""
+#include <cstdio>
+#include <cstdlib>
+#include <vector>
+#include "exact_sum.cuh"
+using namespace sph;
+int main(int argc, char** argv) {
+  const int n = atoi(argv[1]), splits = atoi(argv[2]);
+  std::vector<float> row(1 + 3 * n);
+  while (fread(row.data(), 4, row.size(), stdin) == row.size()) {
+    std::vector<DFAcc> part(splits);
+    for (int i = 0; i < n; ++i)
+      part[i / 4 % splits].add(row[1 + 3 * i], row[2 + 3 * i], row[0], row[3 + 3 * i], 0.f, 0.f);
+    double v;
+    if (splits == 1) {
+      v = part[0].value();
+    } else {
+      SplitSum s(part[0]);
+      for (int k = 1; k < splits; ++k) s.add(SplitSum(part[k]));
+      v = s.value();
+    }
+    fwrite(&v, 8, 1, stdout);
+  }
+  return 0;
+}
+"""
+
 PROGRAM = r"""
 #include <cstdio>
 #include <cstdlib>
@@ -44,17 +73,22 @@ int main(int argc, char** argv) {
 """
 
 
-@pytest.fixture(scope="module")
-def run():
+def _compile(name, program):
     cxx = shutil.which("g++") or shutil.which("c++")
     if cxx is None:
         pytest.skip("no C++ compiler")
     os.makedirs(OUT, exist_ok=True)
-    src, exe = os.path.join(OUT, "probe.cpp"), os.path.join(OUT, "probe")
+    src, exe = os.path.join(OUT, name + ".cpp"), os.path.join(OUT, name)
     with open(src, "w") as fh:
-        fh.write(PROGRAM)
+        fh.write(program)
     subprocess.run([cxx, "-std=c++17", "-O2", "-ffp-contract=off", "-Wall", "-I",
                     os.path.join(ROOT, "paper_2206_14780_gb300", "csrc"), src, "-o", exe], check=True)
+    return exe
+
+
+@pytest.fixture(scope="module")
+def run():
+    exe = _compile("probe", PROGRAM)
 
     def go(terms, splits=1):
         terms = np.ascontiguousarray(terms, np.float32)
@@ -96,6 +130,34 @@ def test_sum_is_no_further_off_than_a_float64_sum(run, factors, splits, seed):
         for row in terms.astype(np.float64):
             plain += np.prod(row)
         assert off <= max(abs(Fraction(float(plain)) - exact), 2 * Fraction(2) ** -53 * abs(exact))
+
+
+@pytest.mark.parametrize("n", [80, 250])
+def test_split_rows_are_no_further_off_than_one_accumulator(n):
+    """Rows of a residual in every number of splits against float64 longer arithmetic: the
+    root mean square error over 2,000 rows, relative to the terms' magnitudes, stays within
+    5% (its own scatter is 1/sqrt(4000) = 1.6%) of one float64-combined accumulator's."""
+    exe = _compile("rows", ROWS)
+    rng = np.random.default_rng(n)
+    count = 2000
+    a = 5.0 * rng.random((count, n)) ** 3
+    hi = a.astype(np.float32)
+    lo = (a - hi).astype(np.float32)
+    k = rng.normal(size=(count, 1)).astype(np.float32)
+    x = (k + 0.1 * rng.normal(size=(count, n))).astype(np.float32)
+    rows = np.concatenate([k, np.stack([hi, lo, x], axis=2).reshape(count, 3 * n)], axis=1).astype(np.float32)
+    coef = hi.astype(np.longdouble) + lo
+    terms = coef * (k.astype(np.longdouble) - x)
+    exact, size = terms.sum(axis=1), np.abs(terms).sum(axis=1)
+    rms = {}
+    for splits in (1, 2, 4, 8):
+        out = subprocess.run([exe, str(n), str(splits)], input=rows.tobytes(), capture_output=True, check=True).stdout
+        got = np.frombuffer(out, np.float64)
+        assert got.size == count
+        rms[splits] = float(np.sqrt(np.mean(((got - exact) / size) ** 2)))
+    assert rms[1] < 2.0 ** -48
+    for splits in (2, 4, 8):
+        assert rms[splits] <= 1.05 * rms[1], rms
 
 
 def test_non_finite_terms_give_what_a_float64_sum_gives(run):
