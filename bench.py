@@ -218,6 +218,20 @@ def apply_traffic(alg_bytes):
         return None, f"unavailable ({type(e).__name__})"
 
 
+# the further legs' objects: 20 KB that no reader of the result line needs
+LEGS = ("ensemble", "precision_study", "sequence", "learned", "apply_forms", "channel", "gaussian", "poiseuille", "cg",
+        "shard")
+
+
+def result_lines(out):
+    """The result line (stdout, a few KB, so that a reader which keeps only the end of the
+    output has all of it) and the further legs' objects (one line on stderr)."""
+    line = {k: v for k, v in out.items() if k not in LEGS}
+    if out.get("learned") and "learned_vs_plain" in out["learned"]:
+        line["learned_vs_plain"] = out["learned"]["learned_vs_plain"]
+    return line, {k: out[k] for k in LEGS if k in out}
+
+
 class ClockSampler:
     """nvidia-smi samples of SM clock and throttle reasons during the timed region."""
 
@@ -596,7 +610,10 @@ def run_sphvisc(args):
                clocks=dict(sm_mhz=clk["sm_mhz"], sm_max_mhz=clk["sm_max_mhz"], reasons=clk["reasons"],
                            samples=clk["samples"]),
                wall_s=wall)
-    print(json.dumps(out))
+    line, legs = result_lines(out)
+    if any(v is not None for v in legs.values()):
+        print(json.dumps(legs), file=sys.stderr)
+    print(json.dumps(line))
     if world > 1:
         import torch.distributed as dist
 
