@@ -192,8 +192,9 @@ def read_peaks():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-# the sources of the operator apply kernel (k_apply_dot and what it includes)
-TRAFFIC_SOURCES = ("tiles.cuh", "solver.cu", "reduce.cuh", "bicgstab_scalars.cuh", "sph_internal.cuh")
+# the sources of the operator apply kernel (k_tile_apply_dot and what it includes) and of
+# the lists it reads, whose order and filling the traffic depends on
+TRAFFIC_SOURCES = ("tiles.cuh", "solver.cu", "neighbors.cu", "reduce.cuh", "bicgstab_scalars.cuh", "sph_internal.cuh")
 
 
 def apply_traffic(alg_bytes):

@@ -249,7 +249,9 @@ typedef struct {
                               dependent launches, each launch processed while its
                               predecessor still runs (default); 1: plain
                               stream-ordered launches.  Same results either way;
-                              sets of up to about 100k particles run as one
+                              sets whose tiles fit one block per SM (rows of ~80
+                              neighbours: up to about 116k particles, thin layers
+                              up to 150k) run as one
                               cooperative kernel under both (BiCGSTAB, direct
                               reductions, apply_form 0, profiling off)            */
   int32_t method;          /* SPH_SOLVER_BICGSTAB (default) or SPH_SOLVER_CG      */

@@ -1017,18 +1017,24 @@ static int region_class(int need, int least) {
 
 // Slices per tile.  Large tiles share more of their neighbours (4.4 union rows per row
 // at 8 slices, 5.8 at 4, 7.8 at 2 on the box); small ones give a small set more blocks
-// and a row more threads.  Whole solves at 8 / 4 / 2 slices in the cooperative kernel
-// (persist.cu): 2.2k rows 837 / 761 / 810 us, 6.8k 1476 / 1392 / 1465, 16k 1865 / 1981 /
-// 2059, 30k 2609 / 2690 / 3162, 51k 3790 / 3543 / 3747; only 8 slices fit at 104k.  Applies of the
-// five-kernel loop: 64k rows 17.3 / 16.5 / 18.0 us, 274k 37.5 / 37.5 / 41.4, 1,157k 128 / 138 / 161.
-// The Gaussian's unions are larger and its rows longer: apply at 190k rows 67.8 / 53.6 /
-// 56.4, but at 77k the cooperative kernel holds 8 slices better (6117 / 7213 us a solve).
-// One slice where that gives fewer tiles than SMs (twice as many with rows of ~250):
-// the set-up kernels' chains per row halve.  Against two slices, us a pass: step of 1.4k
-// rows 890 -> 855, 2.6k 896 -> 812, 4.6k 925 -> 876, solve of 2.7k 1058 -> 990; Gaussian
-// steps of 4.7k, 5.6k, 9.2k rows 1538 -> 1348, 1637 -> 1537, 1367 -> 1214, Gaussian solves
-// 1% either way.  Beyond, two slices are as fast or faster (solve of 6.8k rows 1395 / 1485).
-// 2,400-3,040 slices of ~80 in tiles of 4: 1-10% slower than 8 everywhere.
+// and a row more threads.  Whole passes (rebuild, start, solve to 1e-8) at 8 / 4 / 2 / 1
+// slices, us, all on the cooperative kernel (persist.cu) where it takes them:
+//   rows of ~80    2.2k  1124 /  949 /  896 /  921      rows of ~250
+//                  2.7k  1142 / 1025 / 1010 /  935         3.1k 1487 / 1210 / 1068 / 1034
+//                  6.8k  1626 / 1441 / 1584 / 1499        11.5k 2449 / 1999 / 1880 / 1916
+//                   16k  2142 / 2093 / 2153 / 2117        34.7k 3633 / 3449 / 4219 / 4602
+//                   30k  3160 / 3062 / 3103 / 3345        77.4k 6858 / 7886 / 8528 / 8371
+//                   51k  4173 / 4268 / 4221 / 5721
+//                   59k  4044 / 4195 / 4587 / 6004
+//                   79k  6176 / 6265 / 7150
+//                   97k  6507 / 7636 / 7642
+// (iteration counts differ by up to 5% with the sums' order, which is part of these).  One
+// slice where that gives fewer tiles than SMs (twice as many with rows of ~250), 2 up to
+// 600 slices, 4 up to 1,800, then 8: of the columns above the fastest or within 3% of it,
+// but at 6.8k rows 10% behind 4 slices.  Applies of the five-kernel loop, 8 / 4 / 2: 64k rows
+// 17.3 / 16.5 / 18.0 us, 274k 37.5 / 37.5 / 41.4, 1,157k 128 / 138 / 161; the Gaussian's
+// unions are larger: 190k rows 67.8 / 53.6 / 56.4, hence 4 slices again beyond what the
+// cooperative kernel holds (18 slices per SM).
 // Beyond 320 (640) entries per row the lists of 8 (4) slices exceed the plan's shared
 // memory.
 static int tile_slices_for(int64_t nslices, int32_t maxnb, int num_sms) {

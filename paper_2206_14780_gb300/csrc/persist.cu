@@ -3,10 +3,15 @@
 //
 // Below ~100k rows an iteration of the five-kernel loop (solver.cu) costs 37-50 us of
 // which the applies' memory traffic is a few: the rest is five launches and three
-// grid reductions whose last block runs alone.  Whole solves to 1e-8, five kernels /
-// this one, us: 2.2k rows 1292 / 761, 6.8k 2231 / 1392, 16k 2941 / 1865, 30k 3921 /
-// 2609, 51k 5247 / 3543, 104k 7577 / 6650; Gaussian 12k 2341 / 1620, 35k 4303 / 3040,
-// 77k 6537 / 6120.  What is left per iteration (2.2k rows: 17 us) is the three
+// grid reductions whose last block runs alone.  Whole passes (rebuild, start, solve to
+// 1e-8) at the tile sizes neighbors.cu picks, five kernels / this one, us: 2.2k rows
+// 1386 / 921, 6.8k 2043 / 1584, 16k 2597 / 2153, 30k 3567 / 3062, 51k 5125 / 4268, 59k
+// 5337 / 4044, 79k 6779 / 6269, 97k 7437 / 6552, 110k 7735 / 7463; Gaussian 3.1k 1419 / 1034,
+// 11.5k 2522 / 1880, 35k 4334 / 3449, 77k 8815 / 6858.  Three 8-slice tiles a block reach
+// 116.7k rows; a fourth needs unions below ~1,330 rows, which thin layers have (a slope of
+// 8 spacings, 133k rows: 12601 / 9855) and boxes, channels and deep slopes of that size do
+// not (1,460-1,560: they run the loop, 117k rows 8705, 155k 10378).
+// What is left per iteration (2.2k rows: 17 us) is the three
 // exchanges at ~3 us each and the latency of two applies' streams.  Here one block of 512 threads per SM
 // keeps, for every distinct neighbour of its tiles, r (or r*), p and A p in shared
 // memory (40 bytes with its row number), so that blocks exchange A p and A r* only,
