@@ -115,8 +115,9 @@ typedef struct sph_neighbors sph_neighbors;
  *   positions among the distinct neighbours of a run of rows: about
  *   4 * max_neighbors bytes of device memory per particle with the search's own
  *   copy (520 B at the default 128).  Particle sets too uneven for that, and the
- *   entry points that walk 32-bit rows (export, the on-the-fly apply, features),
- *   take 4 * max_neighbors bytes more.
+ *   entry points that walk 32-bit rows (export, the on-the-fly apply, features, row
+ *   norms, float64 and sharded solves, batches of small scenes), take 4 *
+ *   max_neighbors bytes more.
  * Copies pos/rho/mu/ptype into the handle: the scene arrays may be freed after
  * the call returns.  A rebuild that fails once it has begun (SPH_ERR_CAPACITY,
  * SPH_ERR_NONFINITE, a CUDA error) leaves the handle without lists: calls that need
