@@ -1059,7 +1059,9 @@ sph_status require_lists(const sph_neighbors* H) {
 
 bool stream_capturing(cudaStream_t st) {
   cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(st, &s) == cudaSuccess && s != cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+  (void)cudaGetLastError();   // (the legacy stream while another one captures: what follows fails by itself)
+  return false;
 }
 
 sph_status ensure_nbr(sph_neighbors* H, cudaStream_t st) {
@@ -1067,8 +1069,12 @@ sph_status ensure_nbr(sph_neighbors* H, cudaStream_t st) {
   if (H->nbr_ready) return SPH_OK;
   const bool capturing = stream_capturing(st);
   if (H->nbr_valid && !capturing) {   // expanded by an earlier call, on whatever stream
-    if (cudaEventQuery(H->nbr_event) == cudaSuccess) H->nbr_ready = true;
-    else SPH_TRY_CUDA(cudaStreamWaitEvent(st, H->nbr_event, 0));
+    if (cudaEventQuery(H->nbr_event) == cudaSuccess) {
+      H->nbr_ready = true;
+      return SPH_OK;
+    }
+    (void)cudaGetLastError();   // cudaErrorNotReady is no failure of the next launch
+    SPH_TRY_CUDA(cudaStreamWaitEvent(st, H->nbr_event, 0));
     return SPH_OK;
   }
   SPH_TRY(H->nbr.alloc(H->n_pad * (int64_t)H->maxnb));

@@ -88,10 +88,13 @@ def test_rows_made_on_one_stream_are_read_on_another():
     nb, t = lib_build(s)
     v, y = _velocity(s), torch.zeros((s.n, 4), device="cuda")
     first, second = torch.cuda.Stream(), torch.cuda.Stream()
+    busy = torch.zeros((8192, 8192), device="cuda", dtype=torch.bfloat16)
     for _ in range(5):
         nb.rebuild(t["pos"], t["rho"], t["mu"], t["ptype"], s.lo, s.hi, s.periodic, s.h)
         torch.cuda.synchronize()
         with torch.cuda.stream(first):
+            for _ in range(20):     # the rows are not made yet when the other stream asks
+                busy @ busy
             nb.apply_otf(params_for(s), v, y)
         with torch.cuda.stream(second):
             o, i = nb.export()
