@@ -115,9 +115,9 @@ typedef struct sph_neighbors sph_neighbors;
  *   positions among the distinct neighbours of a run of rows: about
  *   4 * max_neighbors bytes of device memory per particle with the search's own
  *   copy (520 B at the default 128).  Particle sets too uneven for that, and the
- *   entry points that walk 32-bit rows (export, the on-the-fly apply, features, row
- *   norms, float64 and sharded solves, batches of small scenes), take 4 *
- *   max_neighbors bytes more.
+ *   entry points that walk 32-bit rows (export, the on-the-fly apply, features,
+ *   float64 and sharded solves, batches of small scenes), take 4 * max_neighbors
+ *   bytes more.
  * Copies pos/rho/mu/ptype into the handle: the scene arrays may be freed after
  * the call returns.  A rebuild that fails once it has begun (SPH_ERR_CAPACITY,
  * SPH_ERR_NONFINITE, a CUDA error) leaves the handle without lists: calls that need
@@ -658,10 +658,7 @@ sph_status sph_set_row_scale(sph_neighbors* handle, const float* scale, void* st
 /* norm2 (device [n] float, caller order) = squared Euclidean norm of each row of
  * D^-1 A(dt) for params: 1 + sum (a / D)^2 over a fluid row's coefficients, 1 +
  * sum S^2 over a dummy-wall row's Shepard weights, 1 for an identity row
- * (float32 sums of the stored float32 coefficients).  The first call of this,
- * sph_wall_row_scale or sph_mlp_scale_targets after a set-up makes the coefficients
- * along 32-bit rows: it allocates and synchronises, so it comes before a stream
- * capture of one. */
+ * (float32 sums of the stored float32 coefficients). */
 sph_status sph_row_norms(sph_neighbors* handle, const sph_visc_params* params, float* norm2, void* stream);
 
 /* The closed-form wall scale: scale (device [n] float, caller order) =

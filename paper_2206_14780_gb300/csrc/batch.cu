@@ -867,7 +867,7 @@ sph_status sph_batch_create(sph_neighbors* const* handles, const sph_visc_params
       set_error("sph_batch_create: handle %d is null", s);
       return fail(SPH_ERR_INVALID);
     }
-    sph_status e = ensure_operator(H, &params[s], st, Bt->tile_form ? OP_FAST : OP_IH);
+    sph_status e = ensure_operator(H, &params[s], st, Bt->tile_form ? OP_TILE : OP_IH);
     if (e == SPH_OK) e = row_scale_refresh(H, st);
     if (e != SPH_OK) return fail(e);
     Bt->handles.push_back(H);
@@ -1000,7 +1000,7 @@ sph_status sph_batch_solve(sph_batch* Bt, const sph_solve_opts* O, const double*
   for (int s = 0; s < S; ++s) {
     sph_neighbors* H = Bt->handles[s];
     // (a set-up at other parameters and back may have made the other form only)
-    SPH_TRY(ensure_operator(H, &Bt->params[s], st, Bt->tile_form ? OP_FAST : OP_IH));
+    SPH_TRY(ensure_operator(H, &Bt->params[s], st, Bt->tile_form ? OP_TILE : OP_IH));
     scene_view(Bt, H, Bt->hdesc[s]);
     const int64_t o = Bt->row_off[s];
     SPH_LAUNCH(kb_gather, grid_for(H, H->n_pad), kBlock, 0, st)(b[s], H->perm.p, H->n, H->n_pad,

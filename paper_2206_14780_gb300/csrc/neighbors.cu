@@ -833,9 +833,9 @@ __global__ void __launch_bounds__(256) k_tile_plan(const uint8_t* __restrict__ t
 // sums along them does not depend on how the lists were made.  The plan's entries are
 // ordered for shared-memory banks; rows expanded from those cost the export's sort most
 // (rebuild and export of 77k rows of ~250: 7.69 ms against 6.50, 12k: 3.43 against 2.97)
-// and the on-the-fly apply a little (rebuild and apply, 58k rows: 352 against 332 us),
-// while set-ups along 32-bit rows are 3-6% faster on them (rebuild and row norms, 58k:
-// 435 against 452 us).  One block per tile: the region's rows into shared memory, then
+// and the on-the-fly apply a little (rebuild and apply, 58k rows: 352 against 336 us),
+// while applies along stored 32-bit rows are 4% faster on them (58k: 44.5 against 45.9 us
+// an iteration).  One block per tile: the region's rows into shared memory, then
 // one coalesced pass over the entries.
 __global__ void __launch_bounds__(256) k_tile_expand(const uint16_t* __restrict__ raw, const int2* __restrict__ tcells,
                                                      const int32_t* __restrict__ tncell, const int32_t* __restrict__ cnt,

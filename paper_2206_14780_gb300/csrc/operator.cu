@@ -359,11 +359,12 @@ sph_status ensure_operator(sph_neighbors* H, const sph_visc_params* P, cudaStrea
     return SPH_ERR_INVALID;
   }
   SPH_TRY(require_lists(H));
-  const bool tile = form == OP_FAST && H->tile_ok;
+  const bool tile = form != OP_IH && H->tile_ok;
   const bool same = H->op_valid && H->op_params.dt == P->dt && H->op_params.boundary == P->boundary &&
                     H->op_params.mean == P->mean && H->op_mu_version == H->mu_version;
   if (same && (tile ? H->op_tile_valid : H->op_ih_valid)) return SPH_OK;
   if (stream_capturing(st)) {   // it would count as set up before anything has run
+    if (same && form == OP_FAST) return SPH_OK;   // set up in the other form
     set_error("the coefficients for these parameters are not set up, and the stream is capturing: call before the capture");
     return SPH_ERR_CUDA;
   }

@@ -27,33 +27,48 @@ namespace {
 // learned scales are exp(y) with y clamped to this range
 constexpr float kLogScaleMin = -8.f, kLogScaleMax = 2.f;
 
-// squared norm of sorted row s of D^-1 A from the stored float32 coefficients
-__device__ __forceinline__ float row_norm2(const int64_t* __restrict__ off, const int32_t* __restrict__ cnt,
-                                           const int2* __restrict__ ih, const float* __restrict__ invD, int64_t s) {
-  const int2* p = ih + off[s / kSlice] + s % kSlice;
-  const int c = cnt[s];
+// the stored float32 coefficients of the operator, in whichever form it is set up
+struct RowCoefs {
+  const float* hi;        // tile form (tiles.cuh): groups of four entries per lane, filled up with zeros
+  const int64_t* hi_off;
+  const int2* ih;         // SELL-32, where there is no tile form (hi null)
+  const int64_t* ih_off;
+  const int32_t* cnt;
+  const uint8_t* kind;
+  const float* invD;
+};
+
+// squared norm of sorted row s of D^-1 A
+__device__ __forceinline__ float row_norm2(const RowCoefs& R, int64_t s) {
+  const int c = R.cnt[s], lane = (int)(s % kSlice);
   float acc = 0.f;
-  for (int j = 0; j < c; ++j) {
-    const float a = __int_as_float(p[(int64_t)j * kSlice].y);
-    acc = fmaf(a, a, acc);
+  if (R.hi) {
+    const float4* p = reinterpret_cast<const float4*>(R.hi + R.hi_off[s / kSlice]) + lane;
+    for (int g = 0; g < (c + 3) >> 2; ++g) {
+      const float4 a = p[g * kSlice];
+      acc = fmaf(a.w, a.w, fmaf(a.z, a.z, fmaf(a.y, a.y, fmaf(a.x, a.x, acc))));
+    }
+  } else {
+    const int2* p = R.ih + R.ih_off[s / kSlice] + lane;
+    for (int j = 0; j < c; ++j) {
+      const float a = __int_as_float(p[(int64_t)j * kSlice].y);
+      acc = fmaf(a, a, acc);
+    }
   }
-  const float w = invD[s];
+  const float w = R.invD[s];
   return fmaf(w * w, acc, 1.f);
 }
 
 // out[perm[s]] = squared norm of row s of D^-1 A (mode 0), or the wall scale:
 // 1 on fluid and identity rows, factor norm2^-power on Shepard rows (mode 1)
-__global__ void k_row_norms(const int64_t* __restrict__ off, const int32_t* __restrict__ cnt,
-                            const int2* __restrict__ ih, const uint8_t* __restrict__ kind,
-                            const float* __restrict__ invD, const int32_t* __restrict__ perm, int64_t n, int mode,
-                            float factor, float power, float* __restrict__ out) {
+__global__ void k_row_norms(RowCoefs R, const int32_t* __restrict__ perm, int64_t n, int mode, float factor, float power,
+                            float* __restrict__ out) {
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
     float v;
     if (mode == 0) {
-      v = row_norm2(off, cnt, ih, invD, s);
+      v = row_norm2(R, s);
     } else {
-      v = kind[s] == KIND_SHEPARD ? (power != 0.f ? factor * powf(row_norm2(off, cnt, ih, invD, s), -power) : factor)
-                                  : 1.f;
+      v = R.kind[s] == KIND_SHEPARD ? (power != 0.f ? factor * powf(row_norm2(R, s), -power) : factor) : 1.f;
     }
     out[perm[s]] = v;
   }
@@ -61,15 +76,10 @@ __global__ void k_row_norms(const int64_t* __restrict__ off, const int32_t* __re
 
 // training targets of the learned scale: (log of the closed-form wall scale, 0, 0, 0)
 // and the mask of the wall rows (caller order)
-__global__ void k_scale_targets(const int64_t* __restrict__ off, const int32_t* __restrict__ cnt,
-                                const int2* __restrict__ ih, const uint8_t* __restrict__ kind,
-                                const float* __restrict__ invD, const uint8_t* __restrict__ type,
-                                const int32_t* __restrict__ perm, int64_t n, float log_factor, float power,
-                                float4* __restrict__ tgt, uint8_t* __restrict__ mask) {
+__global__ void k_scale_targets(RowCoefs R, const uint8_t* __restrict__ type, const int32_t* __restrict__ perm, int64_t n,
+                                float log_factor, float power, float4* __restrict__ tgt, uint8_t* __restrict__ mask) {
   for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
-    const float t = kind[s] == KIND_SHEPARD
-                        ? log_factor - (power != 0.f ? power * logf(row_norm2(off, cnt, ih, invD, s)) : 0.f)
-                        : 0.f;
+    const float t = R.kind[s] == KIND_SHEPARD ? log_factor - (power != 0.f ? power * logf(row_norm2(R, s)) : 0.f) : 0.f;
     const int64_t i = perm[s];
     tgt[i] = make_float4(t, 0.f, 0.f, 0.f);
     mask[i] = type[s] == SPH_FLUID ? 0 : 1;
@@ -105,11 +115,15 @@ __global__ void k_rs_apply(const float* __restrict__ rs, const int32_t* __restri
   }
 }
 
+RowCoefs row_coefs(const sph_neighbors* H) {
+  const bool tile = H->op_tile_valid;
+  return RowCoefs{tile ? H->t_hi.p : nullptr, H->t_off.p, H->op_ih.p, H->op_off.p, H->op_cnt.p, H->op_kind.p, H->invD.p};
+}
+
 sph_status row_norms_impl(sph_neighbors* H, const sph_visc_params* P, int mode, double factor, double power,
                           float* out, cudaStream_t st) {
-  SPH_TRY(ensure_operator(H, P, st, OP_IH));
-  SPH_LAUNCH(k_row_norms, grid_for(H, H->n), kBlock, 0, st)(H->op_off.p, H->op_cnt.p, H->op_ih.p, H->op_kind.p,
-                                                             H->invD.p, H->perm.p, H->n, mode, (float)factor,
+  SPH_TRY(ensure_operator(H, P, st));
+  SPH_LAUNCH(k_row_norms, grid_for(H, H->n), kBlock, 0, st)(row_coefs(H), H->perm.p, H->n, mode, (float)factor,
                                                              (float)power, out);
   SPH_TRY_CUDA(cudaGetLastError());
   return SPH_OK;
@@ -207,9 +221,8 @@ sph_status sph_mlp_scale_targets(sph_neighbors* h, const sph_visc_params* params
   }
   if (!scale_args_ok("sph_mlp_scale_targets", factor, power)) return SPH_ERR_INVALID;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  SPH_TRY(ensure_operator(h, params, st, OP_IH));
-  SPH_LAUNCH(k_scale_targets, grid_for(h, h->n), kBlock, 0, st)(h->op_off.p, h->op_cnt.p, h->op_ih.p, h->op_kind.p,
-                                                                 h->invD.p, h->type_s.p, h->perm.p, h->n,
+  SPH_TRY(ensure_operator(h, params, st));
+  SPH_LAUNCH(k_scale_targets, grid_for(h, h->n), kBlock, 0, st)(row_coefs(h), h->type_s.p, h->perm.p, h->n,
                                                                  (float)std::log(factor), (float)power,
                                                                  reinterpret_cast<float4*>(targets), mask);
   SPH_TRY_CUDA(cudaGetLastError());

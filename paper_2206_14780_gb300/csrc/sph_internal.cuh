@@ -367,8 +367,10 @@ sph_status visc_apply(sph_neighbors* H, const sph_visc_params* P, const float* v
 sph_status visc_apply_noalloc(sph_neighbors* H, const sph_visc_params* P, const float* v, float* y,
                               cudaStream_t st);
 // A(dt) on the handle: the tile form where the lists have one, else SELL-32 with
-// 32-bit rows; OP_IH asks for the latter whatever the lists are
-enum OpForm { OP_FAST, OP_IH };
+// 32-bit rows; OP_IH asks for the latter whatever the lists are.  While the stream is
+// capturing nothing is set up, and OP_FAST (not OP_TILE) is content with either form:
+// what follows it looks at op_tile_valid.
+enum OpForm { OP_FAST, OP_TILE, OP_IH };
 sph_status ensure_operator(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st, OpForm form = OP_FAST);
 // tiles.cu: coefficients in the tile form; y = A v and the residuals with them
 sph_status tile_fill(sph_neighbors* H, const sph_visc_params* P, cudaStream_t st);

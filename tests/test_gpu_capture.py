@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 
 import scenes
+from oracle import operator as oop
 from sph_testutil import lib_build, oracle_system, params_for, rel_l2, torch_cuda
 
 pytestmark = pytest.mark.gpu
@@ -53,6 +54,50 @@ def test_set_up_inside_a_capture_is_refused():
     g.replay()
     torch.cuda.synchronize()
     assert rel_l2(y.cpu().numpy()[:, :3], want) < 1e-5
+
+
+def test_row_norms_are_captured_after_a_set_up():
+    torch = torch_cuda()
+    s = scenes.lava_box(1, n=12)
+    nb, _ = lib_build(s)
+    nb.setup(params_for(s))
+    got, want = torch.zeros(s.n, device="cuda"), torch.zeros(s.n, device="cuda")
+    g, error = _captured(lambda: nb.row_norms(params_for(s), got))
+    assert error is None
+    g.replay()
+    nb.row_norms(params_for(s), want)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(got.cpu().numpy(), want.cpu().numpy())
+    _, _, A = oracle_system(s)
+    np.testing.assert_allclose(got.cpu().numpy(), oop.row_norms2(A), rtol=2e-5)
+
+
+def test_calls_are_captured_on_either_form_of_the_operator():
+    """After an all-float64 solve the operator is set up along 32-bit rows only."""
+    torch = torch_cuda()
+    from paper_2206_14780_gb300 import binding
+
+    s = scenes.lava_box(1, n=12)
+    nb, t = lib_build(s)
+    x, b = torch.from_numpy(s.x0).cuda(), torch.from_numpy(s.b).cuda()
+    rep = nb.solve(params_for(s), binding.solve_opts(precision=binding.SPH_PREC_FP64), b, x)
+    assert rep["status"] == 0
+    v, y, norms = _velocity(s), torch.zeros((s.n, 4), device="cuda"), torch.zeros(s.n, device="cuda")
+    nb.apply_noalloc(params_for(s), v, y)
+    want = y.clone()
+
+    def calls():
+        nb.apply_noalloc(params_for(s), v, y)
+        nb.row_norms(params_for(s), norms)
+
+    y.zero_()
+    g, error = _captured(calls)
+    assert error is None
+    g.replay()
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(y.cpu().numpy(), want.cpu().numpy())
+    _, _, A = oracle_system(s)
+    np.testing.assert_allclose(norms.cpu().numpy(), oop.row_norms2(A), rtol=2e-5)
 
 
 def test_rows_expanded_inside_a_capture():

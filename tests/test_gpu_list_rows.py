@@ -64,6 +64,9 @@ def test_rows_of_tiles_and_of_the_global_scan(nf):
         nb.apply_otf(params_for(s), torch.from_numpy(v).cuda(), y)
         nb.row_norms(params_for(s), norms)
         got.append((y[:a.n].cpu().numpy(), norms[:a.n].cpu().numpy()))
-    for x, y in zip(*got):
-        assert np.isfinite(x).all()
-        np.testing.assert_array_equal(x, y)
+    (y0, norms0), (y1, norms1) = got
+    assert np.isfinite(y0).all() and np.isfinite(norms0).all()
+    np.testing.assert_array_equal(y0, y1)
+    # the row norms run along the operator's own form: sums of at most ~100 positive float32
+    # terms in another order, 100 half-units of float32's last place
+    np.testing.assert_allclose(norms0, norms1, rtol=100 * 2.0 ** -24)
